@@ -773,15 +773,14 @@ __global__ void __launch_bounds__(kCBlock, sizeof(T) == 4 ? SELM_PATCH_MIN_BLOCK
   const int chunk = (int)(item / ((long long)fy * segs));
   const int q = (int)(col / segs), seg = (int)(col - (long long)q * segs);
   const int m0 = chunk * kc, m1 = min(m0 + kc, fz);
-  const long long plane = (long long)fx * fy;
+  const int plane = fx * fy;
   const int x0 = seg << 3;
-  T* zp = vp + c * G.fsize;
-  const T* rr0 = rp + c * G.fsize;
-  const long long base = (long long)q * fx + x0;
+  // row (m, q, x0) of the correction and of the residual, and its y and x neighbours relative to it
+  T* pv = vp + c * G.fsize + (long long)m0 * plane + q * fx + x0;
+  const T* pr = rp + (pv - vp);
   const int qm = q == 0 ? fy - 1 : q - 1, qp = q == fy - 1 ? 0 : q + 1;
-  const long long ymb = (long long)qm * fx + x0, ypb = (long long)qp * fx + x0;
-  const long long rowx = (long long)q * fx;
-  const int xl_i = x0 == 0 ? fx - 1 : x0 - 1, xr_i = x0 + 8 == fx ? 0 : x0 + 8;
+  const int dym = (qm - q) * fx, dyp = (qp - q) * fx;
+  const int dxl = x0 == 0 ? fx - 1 : -1, dxr = x0 + 8 == fx ? 8 - fx : 8;
   const T sf = (T)G.sf;
   const T w2 = (T)(G.wcf / ((double)G.nch * G.nch));
   const T w1 = (T)(G.wcf / G.nch);
@@ -789,74 +788,72 @@ __global__ void __launch_bounds__(kCBlock, sizeof(T) == 4 ? SELM_PATCH_MIN_BLOCK
   const unsigned long long cy = NOISE ? *cyc : 0ull;
   const uint32_t c1 = ((uint32_t)c << 4) | ((uint32_t)pass << 8) | ((uint32_t)sweep << 12) | (2u << 20);
   T prev[8], cur[8], nxt[8], rr[8], ym[8], yp[8];
+  T rdg = (T)0, rsd = (T)0, dlast = (T)0;   // of the last layer: layers share the diagonal away from the interface
 #pragma unroll
   for (int e = 0; e < 8; ++e) prev[e] = (T)0;
-  if (m0 > 0) Vec<T>::load8(zp + base + (long long)(m0 - 1) * plane, prev);
-  Vec<T>::load8(zp + base + (long long)m0 * plane, cur);
-  for (int m = m0; m < m1; ++m) {
-    const long long mp = (long long)m * plane;
+  if (m0 > 0) Vec<T>::load8(pv - plane, prev);
+  Vec<T>::load8(pv, cur);
+  for (int m = m0; m < m1; ++m, pv += plane, pr += plane) {
     if (m + 1 < fz)
-      Vec<T>::load8(zp + base + mp + plane, nxt);
+      Vec<T>::load8(pv + plane, nxt);
     else {
 #pragma unroll
       for (int e = 0; e < 8; ++e) nxt[e] = (T)0;
     }
-    const int par = (q + m + colour) & 1;
+    const int mpar = (q + m + colour) & 1;
     const bool iface = m == 0 || m == fz - 1;
-    if (!(iface && par)) {
-      Vec<T>::load8(rr0 + base + mp, rr);
-      int nn = 2;
-      T acc[8];
-#pragma unroll
-      for (int e = 0; e < 8; ++e) acc[e] = (m > 0 ? prev[e] : (T)0) + (m + 1 < fz ? nxt[e] : (T)0);
-      nn += (m > 0) + (m + 1 < fz);
-      if (fy > 1) {
-        Vec<T>::load8(zp + ymb + mp, ym);
-        Vec<T>::load8(zp + ypb + mp, yp);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) acc[e] += ym[e] + yp[e];
-        nn += 2;
+    if (!(iface && mpar)) {
+      const T left = pv[dxl], right = pv[dxr];
+      T dg = sf * (T)(2 + (m > 0) + (m + 1 < fz) + (fy > 1 ? 2 : 0));
+      if (iface) dg += w2;
+      T n4[4] = {(T)0, (T)0, (T)0, (T)0};
+      if (NOISE) {
+        const uint32_t grp = (uint32_t)(m * fy + q) * (uint32_t)segs + (uint32_t)seg;
+        Normals<T>::get(philox4x32_10(make_uint4(grp, c1, (uint32_t)cy, (uint32_t)(cy >> 32)), key.k0, key.k1), n4);
       }
-      const T left = zp[rowx + mp + xl_i], right = zp[rowx + mp + xr_i];
-      T dg = sf * (T)nn;
-      T ca[4] = {(T)0, (T)0, (T)0, (T)0};
-      if (iface) {
-        dg += w2;
-        if (m == fz - 1) {
+      if (dg != dlast) {
+        dlast = dg;
+        rsd = NOISE ? (T)1 / tsqrt(dg) : (T)0;
+        rdg = (T)1 / dg;   // one division per row instead of one per site
+      }
+      Vec<T>::load8(pr, rr);
+      ColourSums<T> acc;
+      acc.apply(prev, mpar, [&](T, T x) { return m > 0 ? x : (T)0; });
+      acc.apply(nxt, mpar, [&](T s, T x) { return s + (m + 1 < fz ? x : (T)0); });
+      T s4[4] = {(T)0, (T)0, (T)0, (T)0}, ca[4] = {(T)0, (T)0, (T)0, (T)0};
+      if (fy > 1) {
+        Vec<T>::load8(pv + dym, ym);
+        Vec<T>::load8(pv + dyp, yp);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) ym[e] += yp[e];
+        acc.apply(ym, mpar, [](T s, T x) { return s + x; });
+      }
+      if (iface) {   // the even sites: the late pass takes the odd ones of the interface layers
+        if (fy > 1) {
+          // the siblings in row q ^ 1 (read again: an interface layer is one of fz)
+          Vec<T>::load8(pv + ((q ^ 1) - q) * fx, yp);
+#pragma unroll
+          for (int l = 0; l < 4; ++l) s4[l] = yp[2 * l] + yp[2 * l + 1];
+        }
+        if (m == fz - 1) {   // the four base cells above the segment
           const T* brow = vb + c * G.bsize + ((long long)G.K * G.by + (fy > 1 ? (q >> 1) : 0)) * G.bx + (x0 >> 1);
 #pragma unroll
           for (int l = 0; l < 4; ++l) ca[l] = brow[l];
         }
       }
-      T n4[4] = {(T)0, (T)0, (T)0, (T)0};
-      if (NOISE) {
-        const uint32_t grp = (uint32_t)(((long long)m * fy + q) * segs + seg);
-        Normals<T>::get(philox4x32_10(make_uint4(grp, c1, (uint32_t)cy, (uint32_t)(cy >> 32)), key.k0, key.k1), n4);
-      }
-      const T rsd = NOISE ? (T)1 / tsqrt(dg) : (T)0;
-      const T rdg = (T)1 / dg;   // one division per row instead of one per site
-      const bool up1 = (q ^ 1) == qp;   // which loaded y row holds the siblings' row q ^ 1
-#pragma unroll
-      for (int l = 0; l < 4; ++l) {
-#pragma unroll
-        for (int pp = 0; pp < 2; ++pp) {
-          if (pp != par) continue;
-          const int e = 2 * l + pp;
-          const T xl = e == 0 ? left : cur[e - 1];
-          const T xr = e == 7 ? right : cur[e + 1];
-          T off = -sf * (acc[e] + xl + xr);
-          if (iface) {
-            T sib = cur[e ^ 1];
-            if (fy > 1) sib += up1 ? yp[e] + yp[e ^ 1] : ym[e] + ym[e ^ 1];
-            off += w2 * sib;
-            if (m == fz - 1) off -= w1 * ca[l];
-          }
-          T nv = (rr[e] - off) * rdg;
-          if (NOISE) nv += n4[l] * rsd;
-          cur[e] = nv;
+      colour_update(cur, rr, acc, left, right, mpar, [&](int l, T a, T rv, T xl, T xr, T pair) {
+        T off = -sf * (a + xl + xr);
+        if (iface) {
+          T sib = pair;
+          if (fy > 1) sib += s4[l];
+          off += w2 * sib;
+          if (m == fz - 1) off -= w1 * ca[l];
         }
-      }
-      Vec<T>::store8(zp + base + mp, cur);
+        T nv = (rv - off) * rdg;
+        if (NOISE) nv += n4[l] * rsd;
+        return nv;
+      });
+      Vec<T>::store8(pv, cur);
     }
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
@@ -1036,8 +1033,8 @@ selm_status patch_sweeps_t(selm_comp* C, T* vp, const T* vb, const T* rp, int co
     for (int pass = 0; pass < 4; ++pass) {
       prof::Scope ps(SELM_K_FINE_SWEEP, st);
       const long long rows = (long long)((pass & 1) ? 2 : G.fz) * G.fy * G.ncomp;
-      if (v8 && !(pass & 1)) {   // main pass: march along the layers (chunks of 16)
-        const int kc = 16;
+      if (v8 && !(pass & 1)) {   // main pass: march along the layers
+        const int kc = z_chunk((long long)G.fy * (G.fx >> 3) * G.ncomp, G.fz, (int)sizeof(T));
         const long long nt = (long long)G.fy * (G.fx >> 3) * ((G.fz + kc - 1) / kc) * G.ncomp;
         if (noise)
           k_comp_patch_zm<T, true><<<cgrid(nt), kCBlock, 0, st>>>(G, vp, vb, rp, pass >> 1, s, kc, key, cyc);

@@ -7,6 +7,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <type_traits>
 
 namespace selm {
 
@@ -119,5 +120,76 @@ struct Vec<double> {
     for (int q = 0; q < 4; ++q) *reinterpret_cast<double2*>(p + 2 * q) = make_double2(o[2 * q], o[2 * q + 1]);
   }
 };
+
+// The four sites of parity P of an 8-wide segment: x[2 l + P] (P a compile-time
+// constant folds to registers, a run-time P to selects).
+template <typename T, typename P>
+__device__ __forceinline__ void colour4(const T x[8], P par, T o[4]) {
+#pragma unroll
+  for (int l = 0; l < 4; ++l) o[l] = par ? x[2 * l + 1] : x[2 * l];
+}
+template <typename T, typename P>
+__device__ __forceinline__ void put_colour4(T x[8], P par, const T o[4]) {
+#pragma unroll
+  for (int l = 0; l < 4; ++l) {
+    x[2 * l] = par ? x[2 * l] : o[l];
+    x[2 * l + 1] = par ? o[l] : x[2 * l + 1];
+  }
+}
+// Their x neighbours: x[2 l + P - 1] and x[2 l + P + 1], the segment's ends from left / right.
+template <typename T, typename P>
+__device__ __forceinline__ void colour4_x(const T x[8], T left, T right, P par, T xl[4], T xr[4]) {
+#pragma unroll
+  for (int l = 0; l < 4; ++l) {
+    xl[l] = par ? x[2 * l] : (l == 0 ? left : x[2 * l - 1]);
+    xr[l] = par ? (l == 3 ? right : x[2 * l + 2]) : x[2 * l + 1];
+  }
+}
+// The sums of a z-marching colour pass over an 8-wide row segment: FP32 keeps
+// all eight (the unused half costs less than selecting), FP64 the colour's
+// four, selected on the integer pipe, since the FP64 pipe (two lanes per clock
+// and SM) is what bounds those passes.
+template <typename T>
+struct ColourSums {
+  static constexpr int W = sizeof(T) == 8 ? 4 : 8;
+  T s[W];
+  template <typename F>
+  __device__ __forceinline__ void apply(const T x[8], int par, F f) {   // s[q] = f(s[q], x at q)
+    if constexpr (W == 4) {
+      T x4[4];
+      colour4(x, par, x4);
+#pragma unroll
+      for (int q = 0; q < W; ++q) s[q] = f(s[q], x4[q]);
+    } else {
+#pragma unroll
+      for (int q = 0; q < W; ++q) s[q] = f(s[q], x[q]);
+    }
+  }
+};
+
+// cen[e] = f(l, acc, b, x_left, x_right, x_pair) at the colour's four sites e = 2 l + par of a
+// row segment (x_pair: the other site of the pair 2 l, 2 l + 1).
+template <typename T, typename F>
+__device__ __forceinline__ void colour_update(T cen[8], const T bb[8], const ColourSums<T>& acc, T left, T right,
+                                              int par, F f) {
+  if constexpr (ColourSums<T>::W == 4) {
+    T b4[4], xl[4], xr[4];
+    colour4(bb, par, b4);
+    colour4_x(cen, left, right, par, xl, xr);
+#pragma unroll
+    for (int l = 0; l < 4; ++l) b4[l] = f(l, acc.s[l], b4[l], xl[l], xr[l], par ? xl[l] : xr[l]);
+    put_colour4(cen, par, b4);
+  } else {
+#pragma unroll
+    for (int l = 0; l < 4; ++l) {
+#pragma unroll
+      for (int pp = 0; pp < 2; ++pp) {
+        if (pp != par) continue;
+        const int e = 2 * l + pp;
+        cen[e] = f(l, acc.s[e], bb[e], e == 0 ? left : cen[e - 1], e == 7 ? right : cen[e + 1], cen[e ^ 1]);
+      }
+    }
+  }
+}
 
 }  // namespace selm

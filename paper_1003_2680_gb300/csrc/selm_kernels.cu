@@ -256,22 +256,6 @@ __device__ __forceinline__ double block_sum(double x) {
 // ends are scalar loads.  The whole segment is written back: its
 // other-colour entries are unchanged and are the only entries other threads
 // read during this pass.
-// Updates the four sites of parity P in an 8-wide segment (compile-time
-// indices keep the arrays in registers).
-template <typename T, bool NOISE, int P>
-__device__ __forceinline__ void fine_update8(T cen[8], const T bb[8], const T acc[8], T left, T right, const T n4[4],
-                                             T s, T rdiag, T rsd) {
-#pragma unroll
-  for (int l = 0; l < 4; ++l) {
-    const int e = 2 * l + P;
-    const T xl = e == 0 ? left : cen[e - 1];
-    const T xr = e == 7 ? right : cen[e + 1];
-    T nv = (bb[e] + s * (acc[e] + xl + xr)) * rdiag;   // rdiag = 1 / A_ii of the row
-    if (NOISE) nv += n4[l] * rsd;
-    cen[e] = nv;
-  }
-}
-
 struct RowPass {
   int rstart[kMaxComps + 1];   // first row of each component (rows = ny * nz)
 };
@@ -849,65 +833,58 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? SELM_ZM_MIN_BLOCKS : 
   const int chunk = (int)(item / ((long long)ny * segs));
   const int j = (int)(col / segs), seg = (int)(col - (long long)j * segs);
   const int k0 = chunk * cp.kc, k1 = min(k0 + cp.kc, nz);
-  const long long plane = (long long)nx * ny;
+  const int plane = nx * ny;
   const int x0 = seg << 3;
-  const long long base = c.off + (long long)j * nx + x0;   // (k = 0, j, x0)
-  const long long ym0 = c.off + (long long)(j == 0 ? ny - 1 : j - 1) * nx + x0;
-  const long long yp0 = c.off + (long long)(j == ny - 1 ? 0 : j + 1) * nx + x0;
-  const long long rowx = c.off + (long long)j * nx;
-  const int xl_i = x0 == 0 ? nx - 1 : x0 - 1, xr_i = x0 + 8 == nx ? 0 : x0 + 8;
+  // row (k, j, x0) of v and b, and its y and x neighbours relative to it
+  T* pv = v + c.off + (long long)k0 * plane + j * nx + x0;
+  const T* pb = b + (pv - v);
+  const int dym = (j == 0 ? ny - 1 : -1) * nx, dyp = (j == ny - 1 ? 1 - ny : 1) * nx;
+  const int dxl = x0 == 0 ? nx - 1 : -1, dxr = x0 + 8 == nx ? 8 - nx : 8;
   const T wxm = sep_w1<T>(c, 3), wxp = sep_w1<T>(c, 5), wym = sep_w1<T>(c, 1), wyp = sep_w1<T>(c, 7);
   const unsigned long long cy = NOISE ? *cyc : 0ull;
   const uint32_t c1 = ctr1_of(L.level, c.comp_id, colour, sweep, 0);
   T prev[8], cur[8], nxt[8], bb[8], ty[8];
+  T rdiag = (T)0, rsd = (T)0, dlast = (T)0;   // of the last row: rows share the diagonal away from the walls
 #pragma unroll
   for (int e = 0; e < 8; ++e) prev[e] = (T)0;
-  if (k0 > 0) Vec<T>::load8(v + base + (long long)(k0 - 1) * plane, prev);
-  Vec<T>::load8(v + base + (long long)k0 * plane, cur);
-  for (int k = k0; k < k1; ++k) {
-    const long long kp = (long long)k * plane;
+  if (k0 > 0) Vec<T>::load8(pv - plane, prev);
+  Vec<T>::load8(pv, cur);
+  for (int k = k0; k < k1; ++k, pv += plane, pb += plane) {
     if (k + 1 < nz)
-      Vec<T>::load8(v + base + kp + plane, nxt);
+      Vec<T>::load8(pv + plane, nxt);
     else {
 #pragma unroll
       for (int e = 0; e < 8; ++e) nxt[e] = (T)0;
     }
-    Vec<T>::load8(b + base + kp, bb);
+    Vec<T>::load8(pb, bb);
     const Band7<T> R = band7_row<T>(c, k);
-    T acc[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) acc[e] = (k > 0 ? R.dn * prev[e] : (T)0) + (k + 1 < nz ? R.up * nxt[e] : (T)0);
+    const int par = (j + k + colour) & 1;
+    ColourSums<T> acc;
+    acc.apply(prev, par, [&](T, T x) { return k > 0 ? R.dn * x : (T)0; });
+    acc.apply(nxt, par, [&](T s, T x) { return s + (k + 1 < nz ? R.up * x : (T)0); });
     if (ny > 1) {
-      Vec<T>::load8(v + ym0 + kp, ty);
-#pragma unroll
-      for (int e = 0; e < 8; ++e) acc[e] += R.a * wym * ty[e];
-      Vec<T>::load8(v + yp0 + kp, ty);
-#pragma unroll
-      for (int e = 0; e < 8; ++e) acc[e] += R.a * wyp * ty[e];
+      Vec<T>::load8(pv + dym, ty);
+      acc.apply(ty, par, [&](T s, T x) { return s + R.a * wym * x; });
+      Vec<T>::load8(pv + dyp, ty);
+      acc.apply(ty, par, [&](T s, T x) { return s + R.a * wyp * x; });
     }
-    const T left = v[rowx + kp + xl_i], right = v[rowx + kp + xr_i];
+    const T left = pv[dxl], right = pv[dxr];
     T n4[4] = {(T)0, (T)0, (T)0, (T)0};
     if (NOISE) {
-      const uint32_t grp = (uint32_t)((long long)k * ny + j) * (uint32_t)segs + (uint32_t)seg;
+      const uint32_t grp = (uint32_t)(k * ny + j) * (uint32_t)segs + (uint32_t)seg;
       Normals<T>::get(philox4x32_10(make_uint4(grp, c1, (uint32_t)cy, (uint32_t)(cy >> 32)), key.k0, key.k1), n4);
     }
-    const T rsd = NOISE ? (T)1 / tsqrt(R.diag) : (T)0;
-    const T rdiag = (T)1 / R.diag;   // one division per row instead of one per site
-    const int par = (j + k + colour) & 1;
-#pragma unroll
-    for (int l = 0; l < 4; ++l) {
-#pragma unroll
-      for (int pp = 0; pp < 2; ++pp) {
-        if (pp != par) continue;
-        const int e = 2 * l + pp;
-        const T xl = e == 0 ? left : cur[e - 1];
-        const T xr = e == 7 ? right : cur[e + 1];
-        T nv = (bb[e] - (acc[e] + R.a * (wxm * xl + wxp * xr))) * rdiag;
-        if (NOISE) nv += n4[l] * rsd;
-        cur[e] = nv;
-      }
+    if (R.diag != dlast) {
+      dlast = R.diag;
+      rsd = NOISE ? (T)1 / tsqrt(R.diag) : (T)0;
+      rdiag = (T)1 / R.diag;   // one division per row instead of one per site
     }
-    Vec<T>::store8(v + base + kp, cur);
+    colour_update(cur, bb, acc, left, right, par, [&](int l, T a, T bv, T xl, T xr, T) {
+      T nv = (bv - (a + R.a * (wxm * xl + wxp * xr))) * rdiag;
+      if (NOISE) nv += n4[l] * rsd;
+      return nv;
+    });
+    Vec<T>::store8(pv, cur);
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
       prev[e] = cur[e];
@@ -958,53 +935,45 @@ __device__ __forceinline__ void fine_colour_zm_item(const LevelDev& L, const Col
   const int chunk = (int)(item / ((long long)ny * segs));
   const int j = (int)(col / segs), seg = (int)(col - (long long)j * segs);
   const int k0 = chunk * cp.kc, k1 = min(k0 + cp.kc, nz);
-  const long long plane = (long long)nx * ny;
+  const int plane = nx * ny;
   const int x0 = seg << 3;
-  const long long base = c.off + (long long)j * nx + x0;
-  const long long ym0 = c.off + (long long)(j == 0 ? ny - 1 : j - 1) * nx + x0;
-  const long long yp0 = c.off + (long long)(j == ny - 1 ? 0 : j + 1) * nx + x0;
-  const long long rowx = c.off + (long long)j * nx;
-  const int xl_i = x0 == 0 ? nx - 1 : x0 - 1, xr_i = x0 + 8 == nx ? 0 : x0 + 8;
+  // row (k, j, x0) of v and b, and its y and x neighbours relative to it
+  T* pv = v + c.off + (long long)k0 * plane + j * nx + x0;
+  const T* pb = b + (pv - v);
+  const int dym = (j == 0 ? ny - 1 : -1) * nx, dyp = (j == ny - 1 ? 1 - ny : 1) * nx;
+  const int dxl = x0 == 0 ? nx - 1 : -1, dxr = x0 + 8 == nx ? 8 - nx : 8;
   const uint32_t c1 = ctr1_of(L.level, c.comp_id, colour, sweep, 0);
   const T s = (T)c.s;
   T prev[8], cur[8], nxt[8], bb[8], ty[8];
+  T rdiag = (T)0, rsd = (T)0, dlast = (T)0;   // of the last row: rows share the diagonal away from the walls
 #pragma unroll
   for (int e = 0; e < 8; ++e) prev[e] = (T)0;
-  if (k0 > 0) ldv8<T, CG>(v + base + (long long)(k0 - 1) * plane, prev);
-  ldv8<T, CG>(v + base + (long long)k0 * plane, cur);
-  for (int k = k0; k < k1; ++k) {
-    const long long kp = (long long)k * plane;
+  if (k0 > 0) ldv8<T, CG>(pv - plane, prev);
+  ldv8<T, CG>(pv, cur);
+  for (int k = k0; k < k1; ++k, pv += plane, pb += plane) {
     if (k + 1 < nz)
-      ldv8<T, CG>(v + base + kp + plane, nxt);
+      ldv8<T, CG>(pv + plane, nxt);
     else {
 #pragma unroll
       for (int e = 0; e < 8; ++e) nxt[e] = (T)0;
     }
-    ldv8<T, CG>(b + base + kp, bb);
+    ldv8<T, CG>(pb, bb);
+    const int par = (j + k + colour) & 1;
     // neighbour sums: y-, y+, z-, z+
-    T acc[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) acc[e] = (T)0;
+    const auto add = [](T s, T x) { return s + x; };
+    ColourSums<T> acc{};
     if (ny > 1) {
-      ldv8<T, CG>(v + ym0 + kp, ty);
-#pragma unroll
-      for (int e = 0; e < 8; ++e) acc[e] += ty[e];
-      ldv8<T, CG>(v + yp0 + kp, ty);
-#pragma unroll
-      for (int e = 0; e < 8; ++e) acc[e] += ty[e];
+      ldv8<T, CG>(pv + dym, ty);
+      acc.apply(ty, par, add);
+      ldv8<T, CG>(pv + dyp, ty);
+      acc.apply(ty, par, add);
     }
-    if (k > 0) {
-#pragma unroll
-      for (int e = 0; e < 8; ++e) acc[e] += prev[e];
-    }
-    if (k + 1 < nz) {
-#pragma unroll
-      for (int e = 0; e < 8; ++e) acc[e] += nxt[e];
-    }
-    const T left = ld1<T, CG>(v + rowx + kp + xl_i), right = ld1<T, CG>(v + rowx + kp + xr_i);
+    if (k > 0) acc.apply(prev, par, add);
+    if (k + 1 < nz) acc.apply(nxt, par, add);
+    const T left = ld1<T, CG>(pv + dxl), right = ld1<T, CG>(pv + dxr);
     T n4[4] = {(T)0, (T)0, (T)0, (T)0};
     if (NOISE) {
-      const uint32_t grp = (uint32_t)((long long)k * ny + j) * (uint32_t)segs + (uint32_t)seg;
+      const uint32_t grp = (uint32_t)(k * ny + j) * (uint32_t)segs + (uint32_t)seg;
       Normals<T>::get(philox10(make_uint4(grp, c1, (uint32_t)cy, (uint32_t)(cy >> 32)), key.k0, key.k1), n4);
     }
     const int edges = (k == 0) + (k == nz - 1);
@@ -1012,13 +981,17 @@ __device__ __forceinline__ void fine_colour_zm_item(const LevelDev& L, const Col
     if (c.zkind == kAxisCellDir) dz += (T)edges;
     if (c.zkind == kAxisCellNeu) dz -= (T)edges;
     const T diag = s * ((ny > 1 ? (T)4 : (T)2) + dz);
-    const T rdiag = (T)1 / diag;   // one division per row instead of one per site
-    const T rsd = NOISE ? (T)1 / tsqrt(diag) : (T)0;
-    if (((j + k + colour) & 1) == 0)
-      fine_update8<T, NOISE, 0>(cur, bb, acc, left, right, n4, s, rdiag, rsd);
-    else
-      fine_update8<T, NOISE, 1>(cur, bb, acc, left, right, n4, s, rdiag, rsd);
-    Vec<T>::store8(v + base + kp, cur);
+    if (diag != dlast) {
+      dlast = diag;
+      rdiag = (T)1 / diag;   // one division per row instead of one per site
+      rsd = NOISE ? (T)1 / tsqrt(diag) : (T)0;
+    }
+    colour_update(cur, bb, acc, left, right, par, [&](int l, T a, T bv, T xl, T xr, T) {
+      T nv = (bv + s * (a + xl + xr)) * rdiag;   // rdiag = 1 / A_ii of the row
+      if (NOISE) nv += n4[l] * rsd;
+      return nv;
+    });
+    Vec<T>::store8(pv, cur);
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
       prev[e] = cur[e];
@@ -3094,21 +3067,21 @@ int coop_blocks() {
 // ---------------------------------------------------------------------------
 // Launchers
 // ---------------------------------------------------------------------------
-// Column items of the level-0 z-marching kernels (nx % 8 == 0): chunks of kc
-// z rows, kc halving (down to 4) while fewer than 96K threads would run.
-long long fine_column_pass(const LevelDev& L, ColumnPass* cp) {
+// Column items of the z-marching kernels (nx % 8 == 0): W-wide segments, chunks of
+// z_chunk() z rows.
+template <typename T>
+long long column_pass(const LevelDev& L, int log2w, ColumnPass* cp) {
   long long cols = 0;
   int nzmax = 0;
   for (int ci = 0; ci < L.ncomp; ++ci) {
-    cols += (long long)L.c[ci].ny * (L.c[ci].nx >> 3);
+    cols += (long long)L.c[ci].ny * (L.c[ci].nx >> log2w);
     nzmax = nzmax > L.c[ci].nz ? nzmax : L.c[ci].nz;
   }
-  cp->kc = 16;
-  while (cp->kc > 4 && cols * ((nzmax + cp->kc - 1) / cp->kc) < 96 * 1024) cp->kc /= 2;
+  cp->kc = z_chunk(cols, nzmax, (int)sizeof(T));
   long long items = 0;
   for (int ci = 0; ci < L.ncomp; ++ci) {
     cp->start[ci] = items;
-    items += (long long)L.c[ci].ny * (L.c[ci].nx >> 3) * ((L.c[ci].nz + cp->kc - 1) / cp->kc);
+    items += (long long)L.c[ci].ny * (L.c[ci].nx >> log2w) * ((L.c[ci].nz + cp->kc - 1) / cp->kc);
   }
   cp->start[L.ncomp] = items;
   return items;
@@ -3119,7 +3092,7 @@ cudaError_t launch_smooth(const LevelDev& L, T* v, const T* b, int sweep, bool n
                           const unsigned long long* cyc, cudaStream_t st) {
   if (L.level == 0 && L.c[0].nx % 8 == 0) {
     ColumnPass cp{};
-    const long long items = fine_column_pass(L, &cp);
+    const long long items = column_pass<T>(L, 3, &cp);
     for (int colour = 0; colour < 2; ++colour) {
       prof::Scope ps(SELM_K_FINE_SWEEP, st);
       if (noise)
@@ -3149,15 +3122,9 @@ cudaError_t launch_smooth(const LevelDev& L, T* v, const T* b, int sweep, bool n
     return cudaGetLastError();
   }
   if (L.rb && L.c[0].nx % 8 == 0) {
-    // banded 7-point level: march along z (chunks of 16 rows)
+    // banded 7-point level: march along z
     ColumnPass cp{};
-    cp.kc = 16;
-    long long items = 0;
-    for (int ci = 0; ci < L.ncomp; ++ci) {
-      cp.start[ci] = items;
-      items += (long long)L.c[ci].ny * (L.c[ci].nx >> 3) * ((L.c[ci].nz + cp.kc - 1) / cp.kc);
-    }
-    cp.start[L.ncomp] = items;
+    const long long items = column_pass<T>(L, 3, &cp);
     for (int colour = 0; colour < 2; ++colour) {
       prof::Scope ps(SELM_K_COARSE_SWEEP, st);
       if (noise)
@@ -3226,19 +3193,13 @@ cudaError_t launch_residual(const LevelDev& L, const T* v, const T* b, T* t, cud
   prof::Scope ps(SELM_K_RESIDUAL, st);
   if (L.level == 0 && L.c[0].nx % 8 == 0) {
     ColumnPass cp{};
-    const long long items = fine_column_pass(L, &cp);
+    const long long items = column_pass<T>(L, 3, &cp);
     LTRY(launch_pdl(k_fine_residual_zm<T>, grid_for(items), kBlock, st, L, cp, v, b, t));
     return cudaGetLastError();
   }
   if (L.rb && L.c[0].nx % 8 == 0) {
     ColumnPass cp{};
-    cp.kc = 16;
-    long long items = 0;
-    for (int ci = 0; ci < L.ncomp; ++ci) {
-      cp.start[ci] = items;
-      items += (long long)L.c[ci].ny * (L.c[ci].nx >> 3) * ((L.c[ci].nz + cp.kc - 1) / cp.kc);
-    }
-    cp.start[L.ncomp] = items;
+    const long long items = column_pass<T>(L, 3, &cp);
     LTRY(launch_pdl(k_band7_residual_zm<T>, grid_for(items), kBlock, st, L, cp, v, b, t));
     return cudaGetLastError();
   }

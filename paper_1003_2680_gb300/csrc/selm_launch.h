@@ -13,6 +13,38 @@ struct Key {
   uint32_t k0, k1;
 };
 
+// z rows per thread (1, 2, 4, 8 or 16) of a z-marching colour pass or residual
+// over `cols` columns of `nz` rows.  A chunk reads two rows more than it
+// updates, and a thread works through its rows one memory latency after the
+// other, so a level that cannot fill the GPU wants short chunks.
+// FP32: the chunk with the least waves x (rows + 2), a wave being the 152 x 768
+// threads that the register budget (three blocks of 256 per SM) keeps
+// resident.  Fixed chunks of 16 on the composite levels, and 4..16 rows for
+// at least 96 K threads on level 0, left most SMs idle on small levels and
+// 192^3 in 1.4 waves: composite FAC cycle at 32^3 + 4 rows 267 -> 177 us, 80^3 +
+// 9 rows 564 -> 420 us; level-0 sweep at 192^3 102 -> 89 us, 128^3 unchanged
+// (29 us, the same chunk).
+// FP64: the FP64 pipe bounds a full GPU whatever the chunk (128^3: 166 us a
+// sweep at 4 and at 8 rows), so the longest chunk that still runs 96 K threads;
+// 64^3: 33 us at 1 row, 37 at 2, 52 at 4; 96^3: 81 us at 2 rows, 90 at 4.
+inline int z_chunk(long long cols, int nz, int esize) {
+  auto threads = [&](int kc) { return cols * ((nz + kc - 1) / kc); };
+  int best = 16;
+  if (esize == 8) {
+    while (best > 1 && threads(best) < 96 * 1024) best /= 2;
+    return best;
+  }
+  long long cost = -1;
+  for (int kc = 16; kc >= 1; kc /= 2) {
+    const long long wave = 152 * 768, t = (threads(kc) + wave - 1) / wave * (kc + 2);
+    if (cost < 0 || t < cost) {
+      cost = t;
+      best = kc;
+    }
+  }
+  return best;
+}
+
 // Stage kernels.  `T` is float or double (inner precision); all launches go
 // on `st`.  Counters (`cyc`) are read from device memory so that the calls can
 // be captured in CUDA graphs.
