@@ -304,7 +304,8 @@ selm_status vcycle_t(selm_mg* h, Sys& s, int l, T* v0, const T* b0, bool noise, 
     const LevelDev& Lc = s.lev[l + 1];
     CK(launch_residual<T>(L, v, b, (T*)s.t[l], st));
     CK(launch_restrict<T>(L, Lc, (const T*)s.t[l], (T*)s.b[l + 1], st));
-    CK(cudaMemsetAsync(s.v[l + 1], 0, (size_t)Lc.size * sizeof(T), st));
+    if (!(s.use_engine && eng.valid && l + 1 == eng.params.l0))   // the engine starts from v = 0 itself
+      CK(cudaMemsetAsync(s.v[l + 1], 0, (size_t)Lc.size * sizeof(T), st));
     selm_status r = vcycle_t<T>(h, s, l + 1, v0, b0, noise, cyc, st);
     if (r != SELM_OK) return r;
     CK(launch_prolong<T>(L, Lc, v, (const T*)s.v[l + 1], st));
@@ -689,10 +690,10 @@ selm_status create_with_host(const selm_mg_desc& d, const HostSystem& host, int 
   const int first = engine_first_level(h, h->vel);
   if (h->esize == 4)
     plan_coarse_engine<float>(h->vel.lev, h->vel.levels, h->vel.b, h->vel.v, h->vel.t, h->vel.eng_dev, st,
-                              &h->vel.engf, 0, first);
+                              &h->vel.engf, h->mu1 + h->mu2, 0, first);
   else
     plan_coarse_engine<double>(h->vel.lev, h->vel.levels, h->vel.b, h->vel.v, h->vel.t, h->vel.eng_dev, st,
-                               &h->vel.engd, 0, first);
+                               &h->vel.engd, h->mu1 + h->mu2, 0, first);
   cudaGetLastError();   // without a plan the per-pass path runs
   *extra_off = xoff;
   *out = h;
@@ -712,10 +713,10 @@ selm_status replan_engine(selm_mg* h, int cluster, cudaStream_t st) {
     sy->engine_cluster = cluster;
     // without a plan (returns false) the per-pass path runs
     if (h->esize == 4)
-      plan_coarse_engine<float>(sy->lev, sy->levels, sy->b, sy->v, sy->t, sy->eng_dev, st, &sy->engf, cluster,
+      plan_coarse_engine<float>(sy->lev, sy->levels, sy->b, sy->v, sy->t, sy->eng_dev, st, &sy->engf, h->mu1 + h->mu2, cluster,
                                 engine_first_level(h, *sy));
     else
-      plan_coarse_engine<double>(sy->lev, sy->levels, sy->b, sy->v, sy->t, sy->eng_dev, st, &sy->engd, cluster,
+      plan_coarse_engine<double>(sy->lev, sy->levels, sy->b, sy->v, sy->t, sy->eng_dev, st, &sy->engd, h->mu1 + h->mu2, cluster,
                                  engine_first_level(h, *sy));
     cudaGetLastError();
   }
@@ -813,9 +814,9 @@ selm_status selm_mg_create(const selm_mg_desc* desc, void* stream, selm_mg** out
     sy->eng_dev = dp;
     const int first = engine_first_level(h, *sy);
     if (h->esize == 4)
-      plan_coarse_engine<float>(sy->lev, sy->levels, sy->b, sy->v, sy->t, dp, st, &sy->engf, 0, first);
+      plan_coarse_engine<float>(sy->lev, sy->levels, sy->b, sy->v, sy->t, dp, st, &sy->engf, h->mu1 + h->mu2, 0, first);
     else
-      plan_coarse_engine<double>(sy->lev, sy->levels, sy->b, sy->v, sy->t, dp, st, &sy->engd, 0, first);
+      plan_coarse_engine<double>(sy->lev, sy->levels, sy->b, sy->v, sy->t, dp, st, &sy->engd, h->mu1 + h->mu2, 0, first);
     cudaGetLastError();
   }
   h->u = (double*)(h->ws + p.u_off);
@@ -1451,10 +1452,10 @@ selm_status static_setup(StaticSlot& slot, const selm_mg_desc& d, cudaStream_t s
   // CUDA error while planning is an error.
   if (h->esize == 4)
     plan_coarse_engine<float>(h->vel.lev, h->vel.levels, h->vel.b, h->vel.v, h->vel.t, h->vel.eng_dev, st,
-                              &h->vel.engf, 0, first);
+                              &h->vel.engf, h->mu1 + h->mu2, 0, first);
   else
     plan_coarse_engine<double>(h->vel.lev, h->vel.levels, h->vel.b, h->vel.v, h->vel.t, h->vel.eng_dev, st,
-                               &h->vel.engd, 0, first);
+                               &h->vel.engd, h->mu1 + h->mu2, 0, first);
   ce = cudaStreamSynchronize(st);
   if (ce == cudaSuccess) ce = cudaGetLastError();
   if (ce != cudaSuccess) {

@@ -18,6 +18,15 @@
 // The visiting order (colour classes in increasing id, all sites of a class
 // updated together) and the Philox streams are those of the per-pass kernels,
 // so both paths produce the same chain.
+//
+// What bounds it: latency.  A pass is a barrier, a site's 45 shared loads and
+// its sum, and about 150 passes follow one another.  So a level's constants
+// sit in registers, everything about a site but the values v is loaded before
+// the barrier that releases its pass, and the normals of a noisy launch are
+// drawn once at its start.  64^3 velocity V-cycle (levels of 32^3 and below),
+// one launch: 157 -> 128 us, noisy 211 -> 174 us; a pass of the 32^3 level 1.15
+// -> 0.81 us; residual of the 16^3 level in CTA 0 9.9 -> 3.1 us, prolongation
+// from it 9.8 -> 4.1 us.
 
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
@@ -29,6 +38,7 @@
 #include "selm_coarse.h"
 #include "selm_internal.h"
 #include "selm_devmath.h"
+#include "selm_pdl.h"
 #include "selm_prof.h"
 
 namespace cg = cooperative_groups;
@@ -36,12 +46,14 @@ namespace cg = cooperative_groups;
 namespace selm {
 namespace {
 
-// Threads per CTA: 512, which leaves up to 128 registers a thread for the
-// unrolled 45-point row (at 1024 threads the 64-register cap spills it and
-// the colour passes on the engine's levels run slower).
+// Threads per CTA.  FP32: 512, which leaves up to 128 registers a thread for
+// the unrolled 45-point row (at 1024 threads the 64-register cap spills it and
+// the colour passes on the engine's levels run slower).  FP64: 256; a row
+// takes twice the registers, and the FP64 pipe (two lanes per clock) is busy
+// with eight warps.
 template <typename T>
 struct EngThreads {
-  static constexpr int value = 512;
+  static constexpr int value = sizeof(T) == 4 ? 512 : 256;
 };
 
 __device__ __forceinline__ uint4 eng_philox10(uint4 c, uint32_t k0, uint32_t k1) { return philox4x32_10(c, k0, k1); }
@@ -109,57 +121,6 @@ __device__ __forceinline__ View<T> make_view(const EngLevel<T>& L, unsigned char
   return w;
 }
 
-// Row of A applied to v in the separable form: for each z offset, two 3x3
-// partial sums with the level's x/y weights, combined with the row's z bands.
-// centre == false excludes the diagonal term (sum_{j != i} A_ij v_j).
-template <typename T, bool CENTRE>
-__device__ __forceinline__ T stencil_row(const View<T>& w, int i, int j, int k) {
-  const EngLevel<T>& L = *w.L;
-  const int nx = L.nx, ny = L.ny, rp = L.rp;
-  const int xm = xpos(i == 0 ? nx - 1 : i - 1, L.half), xp = xpos(i == nx - 1 ? 0 : i + 1, L.half);
-  const int x0 = xpos(i, L.half);
-  const T* zb = w.tab + k * 12;
-  // Planes beyond a wall have zero band weights: their loads are clamped to
-  // a valid plane (inside the slab and its halo) and multiplied by 0, so the
-  // loads of all planes issue without a branch between them.
-  T acc = (T)0;
-#pragma unroll
-  for (int dz = -2; dz <= 2; ++dz) {
-    const int kk = min(max(k + dz, 0), L.nz - 1);
-    const T* vp = w.v + (kk - w.z0 + 2) * L.pp;
-    T p1, p2;
-    if (ny == 1) {
-      const T a = vp[xm], c = vp[xp];
-      p1 = L.w1[3] * a + L.w1[5] * c;
-      p2 = L.w2[3] * a + L.w2[5] * c;
-      if (CENTRE || dz != 0) {
-        const T b = vp[x0];
-        p1 += L.w1[4] * b;
-        p2 += L.w2[4] * b;
-      }
-    } else {
-      const int jm = j == 0 ? ny - 1 : j - 1, jp = j == ny - 1 ? 0 : j + 1;
-      const T* r0 = vp + jm * rp;
-      const T* r1 = vp + j * rp;
-      const T* r2 = vp + jp * rp;
-      const T a0 = r0[xm], b0 = r0[x0], c0 = r0[xp];
-      const T a1 = r1[xm], c1 = r1[xp];
-      const T a2 = r2[xm], b2 = r2[x0], c2 = r2[xp];
-      p1 = L.w1[0] * a0 + L.w1[1] * b0 + L.w1[2] * c0 + L.w1[3] * a1 + L.w1[5] * c1 + L.w1[6] * a2 +
-           L.w1[7] * b2 + L.w1[8] * c2;
-      p2 = L.w2[0] * a0 + L.w2[1] * b0 + L.w2[2] * c0 + L.w2[3] * a1 + L.w2[5] * c1 + L.w2[6] * a2 +
-           L.w2[7] * b2 + L.w2[8] * c2;
-      if (CENTRE || dz != 0) {
-        const T b1 = r1[x0];
-        p1 += L.w1[4] * b1;
-        p2 += L.w2[4] * b1;
-      }
-    }
-    acc += zb[dz + 2] * p1 + zb[5 + dz + 2] * p2;
-  }
-  return acc;
-}
-
 // q = n / d for 0 <= n < 2^24: float reciprocal estimate, then exact correction.
 __device__ __forceinline__ int fdiv(int n, int d, float inv) {
   int q = (int)((float)n * inv);
@@ -168,72 +129,246 @@ __device__ __forceinline__ int fdiv(int n, int d, float inv) {
   return q;
 }
 
-struct Sync {
-  bool cluster;
-  __device__ __forceinline__ void operator()() const {
-    if (cluster)
-      cg::this_cluster().sync();
-    else
-      __syncthreads();
+// A level's constants in registers: the passes read them at every site, and
+// the compiler cannot keep shared-memory values across the stores of v.
+template <typename T>
+struct LevReg {
+  int nx, ny, mx, my, mz, half, rp, pp, z0, ncol, P;
+  int xlast;        // position of x = nx - 1 in a row
+  T* v;             // plane z0 of the slab
+  const T* tab;
+  const EngColour* col;
+  T w1[9], w2[9];
+  __device__ __forceinline__ explicit LevReg(const View<T>& w) {
+    const EngLevel<T>& L = *w.L;
+    nx = L.nx; ny = L.ny; mx = L.mx; my = L.my; mz = L.mz;
+    half = L.half; rp = L.rp; pp = L.pp; z0 = w.z0; ncol = L.ncol; P = L.P;
+    xlast = xpos(L.nx - 1, L.half);
+    v = w.v + 2 * pp;
+    tab = w.tab;
+    col = w.col;
+#pragma unroll
+    for (int q = 0; q < 9; ++q) {
+      w1[q] = L.w1[q];
+      w2[q] = L.w2[q];
+    }
   }
 };
 
-// One colour pass of the stochastic Gauss-Seidel sweep on the owned planes:
-// one thread per site; the four sites of a noise group each recompute the
-// group's Philox block (cheaper than serialising their updates).  Class
-// geometry, z bands, inverse diagonals and noise scales come from the
-// shared-memory tables staged for the level.
-template <typename T, bool NOISE>
-__device__ void colour_pass(const View<T>& w, int level, int q, int sweep, const T* b, bool b_local, int boff, Key key,
-                            unsigned long long cyc, int rank, int csize, bool cluster) {
-  const EngLevel<T>& L = *w.L;
-  const EngColour cc = w.col[q];
-  if (cc.nsite <= 0) return;
-  const uint32_t c1 = (uint32_t)level | ((uint32_t)L.comp_id << 4) | ((uint32_t)q << 8) | ((uint32_t)sweep << 12);
-  cg::cluster_group cl = cg::this_cluster();
-  for (int s = threadIdx.x; s < cc.nsite; s += blockDim.x) {
-    const int rk = cc.rank_lo + s;
-    int t, ii, kk, jj;
-    if (cc.sx >= 0) {
-      t = rk >> cc.sx;
-      ii = rk & (cc.nxc - 1);
+// Positions, within a plane of the slab, of the 3 x 3 window around (i, j)
+// (D2: the three sites of the one row): index (dy + 1) * 3 + dx + 1.
+template <typename T, bool D2>
+__device__ __forceinline__ void window_of(const LevReg<T>& R, int i, int j, int c[9]) {
+  const int h = i >> 1;
+  const int x0 = (i & 1) ? R.half + h : h;
+  const int xm = i == 0 ? R.xlast : ((i & 1) ? h : R.half + h - 1);
+  const int xp = i == R.nx - 1 ? 0 : ((i & 1) ? h + 1 : R.half + h);
+  const int r1 = D2 ? 0 : j * R.rp;
+  c[3] = r1 + xm; c[4] = r1 + x0; c[5] = r1 + xp;
+  if (!D2) {
+    const int r0 = (j == 0 ? R.ny - 1 : j - 1) * R.rp, r2 = (j == R.ny - 1 ? 0 : j + 1) * R.rp;
+    c[0] = r0 + xm; c[1] = r0 + x0; c[2] = r0 + xp;
+    c[6] = r2 + xm; c[7] = r2 + x0; c[8] = r2 + xp;
+  }
+}
+
+// The two x-y partial sums w1 . v and w2 . v of one plane (separable form of
+// the Galerkin row); CENTRE == false leaves out the site itself.
+template <typename T, bool D2, bool CENTRE>
+__device__ __forceinline__ void plane_sums(const LevReg<T>& R, const T* vp, const int c[9], T* s1, T* s2) {
+  T p1, p2;
+  if (D2) {
+    const T a = vp[c[3]], d = vp[c[5]];
+    p1 = R.w1[3] * a + R.w1[5] * d;
+    p2 = R.w2[3] * a + R.w2[5] * d;
+  } else {
+    const T a0 = vp[c[0]], b0 = vp[c[1]], c0 = vp[c[2]];
+    const T a1 = vp[c[3]], c1 = vp[c[5]];
+    const T a2 = vp[c[6]], b2 = vp[c[7]], c2 = vp[c[8]];
+    p1 = R.w1[0] * a0 + R.w1[1] * b0 + R.w1[2] * c0 + R.w1[3] * a1 + R.w1[5] * c1 + R.w1[6] * a2 + R.w1[7] * b2 +
+         R.w1[8] * c2;
+    p2 = R.w2[0] * a0 + R.w2[1] * b0 + R.w2[2] * c0 + R.w2[3] * a1 + R.w2[5] * c1 + R.w2[6] * a2 + R.w2[7] * b2 +
+         R.w2[8] * c2;
+  }
+  if (CENTRE) {
+    const T b1 = vp[c[4]];
+    p1 += R.w1[4] * b1;
+    p2 += R.w2[4] * b1;
+  }
+  *s1 = p1;
+  *s2 = p2;
+}
+
+// Row k of the staged table: 10 z-band entries, 1/A_ii, 1/sqrt(A_ii).
+__device__ __forceinline__ void row_table(const float* tab, int k, float t[12]) {
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    const float4 a = *reinterpret_cast<const float4*>(tab + 12 * k + 4 * q);
+    t[4 * q] = a.x; t[4 * q + 1] = a.y; t[4 * q + 2] = a.z; t[4 * q + 3] = a.w;
+  }
+}
+__device__ __forceinline__ void row_table(const double* tab, int k, double t[12]) {
+#pragma unroll
+  for (int q = 0; q < 6; ++q) {
+    const double2 a = *reinterpret_cast<const double2*>(tab + 12 * k + 2 * q);
+    t[2 * q] = a.x; t[2 * q + 1] = a.y;
+  }
+}
+
+// Everything one site's update needs but the values v: its window, its row
+// of the table, b and its normal.  None of it depends on the passes before,
+// so it is formed between a pass's arrival at the barrier and its release.
+template <typename T>
+struct Site {
+  bool on;
+  int kz;          // plane within the slab
+  int c[9];
+  T row[12], b, n;
+};
+
+template <typename T>
+struct PassArgs {
+  int level, first;            // sweep index of the first pass
+  const T* b;
+  bool b_local;
+  int boff;
+  const T* noise;              // normals of every sweep, or null: formed here
+  int nstride;                 // normals per sweep
+  uint32_t c1;                 // level and component of the noise counter
+  Key key;
+  unsigned long long cyc;
+};
+
+template <typename T, bool NOISE, bool D2>
+__device__ __forceinline__ void load_site(const LevReg<T>& R, const PassArgs<T>& A, const EngColour& cc, int q,
+                                          int sweep, int s, Site<T>& x) {
+  x.on = s < cc.nsite;
+  if (!x.on) return;
+  const int rk = cc.rank_lo + s;
+  int t, ii, kk, jj;
+  if (cc.sx >= 0) {
+    t = rk >> cc.sx;
+    ii = rk & (cc.nxc - 1);
+  } else {
+    t = fdiv(rk, cc.nxc, cc.inv_nxc);
+    ii = rk - t * cc.nxc;
+  }
+  if (cc.sy >= 0) {
+    kk = t >> cc.sy;
+    jj = t & (cc.nyc - 1);
+  } else {
+    kk = fdiv(t, cc.nyc, cc.inv_nyc);
+    jj = t - kk * cc.nyc;
+  }
+  const int i = cc.cx + R.mx * ii, j = cc.cy + R.my * jj, k = cc.cz + R.mz * kk;
+  x.kz = k - R.z0;
+  const int gidx = (k * R.ny + j) * R.nx + i;
+  x.b = A.b_local ? A.b[gidx - A.boff] : ld_cg(A.b + gidx);
+  if (NOISE) {
+    if (A.noise) {
+      x.n = A.noise[sweep * A.nstride + cc.noff + s];
     } else {
-      t = fdiv(rk, cc.nxc, cc.inv_nxc);
-      ii = rk - t * cc.nxc;
-    }
-    if (cc.sy >= 0) {
-      kk = t >> cc.sy;
-      jj = t & (cc.nyc - 1);
-    } else {
-      kk = fdiv(t, cc.nyc, cc.inv_nyc);
-      jj = t - kk * cc.nyc;
-    }
-    const int i = cc.cx + L.mx * ii, j = cc.cy + L.my * jj, k = cc.cz + L.mz * kk;
-    const int gidx = (k * L.ny + j) * L.nx + i;
-    const T bb = b_local ? b[gidx - boff] : ld_cg(b + gidx);
-    const T* tr = w.tab + k * 12;
-    const T off = stencil_row<T, false>(w, i, j, k);
-    T nv = (bb - off) * tr[10];
-    if (NOISE) {
-      T nn;
-      normal_of(eng_philox10(make_uint4((uint32_t)(rk >> 2), c1, (uint32_t)cyc, (uint32_t)(cyc >> 32)), key.k0,
-                             key.k1),
-                rk & 3, &nn);
-      nv += nn * tr[11];
-    }
-    w.v[w.loc(i, j, k)] = nv;
-    if (cluster && csize > 1) {
-      // push into the halos of the CTAs owning planes within distance 2
-      const int rlo = max(0, (k - 2) / L.P), rhi = min(csize - 1, (k + 2) / L.P);
-      for (int r2 = rlo; r2 <= rhi; ++r2) {
-        if (r2 == rank) continue;
-        const int z0b = min(r2 * L.P, L.nz), z1b = min(z0b + L.P, L.nz);
-        if (z0b >= z1b || k < z0b - 2 || k >= z1b + 2) continue;
-        T* rem = cl.map_shared_rank(w.v, r2);
-        rem[(k - z0b + 2) * L.pp + j * L.rp + xpos(i, L.half)] = nv;
-      }
+      normal_of(eng_philox10(make_uint4((uint32_t)(rk >> 2), A.c1 | ((uint32_t)q << 8) | ((uint32_t)sweep << 12),
+                                        (uint32_t)A.cyc, (uint32_t)(A.cyc >> 32)),
+                             A.key.k0, A.key.k1),
+                rk & 3, &x.n);
     }
   }
+  window_of<T, D2>(R, i, j, x.c);
+  row_table(R.tab, k, x.row);
+}
+
+// The heat-bath update of a loaded site.  The planes beyond a wall are the
+// slab's zeroed halo planes and carry zero band weights.
+template <typename T, bool NOISE, bool D2>
+__device__ __forceinline__ T site_value(const LevReg<T>& R, const Site<T>& x) {
+  const T* vp = R.v + x.kz * R.pp;
+  T acc = (T)0;
+#pragma unroll
+  for (int dz = -2; dz <= 2; ++dz) {
+    T p1, p2;
+    if (dz == 0)
+      plane_sums<T, D2, false>(R, vp, x.c, &p1, &p2);
+    else
+      plane_sums<T, D2, true>(R, vp + dz * R.pp, x.c, &p1, &p2);
+    acc += x.row[dz + 2] * p1 + x.row[5 + dz + 2] * p2;
+  }
+  T nv = (x.b - acc) * x.row[10];
+  if (NOISE) nv += x.n * x.row[11];
+  return nv;
+}
+
+// Slabs of the CTAs at distance 1 and 2 (null: none, or the slab is empty).
+template <typename T>
+struct Remote {
+  T* v[4];   // rank - 2, - 1, + 1, + 2: their plane z0, expressed from this CTA's plane z0
+};
+
+// `count` sweeps of a level: every colour class in turn, one thread per site,
+// a barrier after each class.  In the cluster a site within two planes of
+// another slab is also stored into that slab's halo.  The next pass's site
+// is loaded between arrival and release of the barrier.
+template <typename T, bool NOISE, bool D2>
+__device__ void sweeps(const View<T>& w, const PassArgs<T>& A, int count, int rank, int csize, bool cluster) {
+  const LevReg<T> R(w);
+  Remote<T> rem;
+  if (cluster) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int d = q < 2 ? q - 2 : q - 1, r2 = rank + d;
+      rem.v[q] = nullptr;
+      if (r2 >= 0 && r2 < csize && min(r2 * R.P, w.L->nz) < min((r2 + 1) * R.P, w.L->nz))
+        rem.v[q] = cg::this_cluster().map_shared_rank(R.v, r2) - (long long)d * R.P * R.pp;
+    }
+  }
+  const int npass = count * R.ncol;
+  auto update = [&](const Site<T>& x) {
+    const T nv = site_value<T, NOISE, D2>(R, x);
+    const int pos = x.kz * R.pp + x.c[4];
+    R.v[pos] = nv;
+    if (cluster) {
+      // slab rank + d holds this plane when it is within two planes of it
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int d = q < 2 ? q - 2 : q - 1;
+        const bool near = d < 0 ? x.kz < 2 + (d + 1) * R.P : x.kz >= d * R.P - 2;
+        if (rem.v[q] && near) rem.v[q][pos] = nv;
+      }
+    }
+  };
+  int q = 0, sweep = A.first;
+  EngColour cc = R.col[0];
+  Site<T> x;
+  load_site<T, NOISE, D2>(R, A, cc, 0, sweep, threadIdx.x, x);
+  for (int p = 0; p < npass; ++p) {
+    if (x.on) update(x);
+    for (int s = threadIdx.x + blockDim.x; s < cc.nsite; s += blockDim.x) {
+      load_site<T, NOISE, D2>(R, A, cc, q, sweep, s, x);
+      update(x);
+    }
+    if (cluster) cg::this_cluster().barrier_arrive();
+    if (++q == R.ncol) {
+      q = 0;
+      ++sweep;
+    }
+    if (p + 1 < npass) {
+      cc = R.col[q];
+      load_site<T, NOISE, D2>(R, A, cc, q, sweep, threadIdx.x, x);
+    }
+    if (cluster)
+      cg::this_cluster().barrier_wait();
+    else
+      __syncthreads();
+  }
+}
+
+template <typename T, bool NOISE>
+__device__ __forceinline__ void sweeps_any(const View<T>& w, const PassArgs<T>& A, int count, int rank, int csize,
+                                           bool cluster) {
+  if (w.L->ny == 1)
+    sweeps<T, NOISE, true>(w, A, count, rank, csize, cluster);
+  else
+    sweeps<T, NOISE, false>(w, A, count, rank, csize, cluster);
 }
 
 template <typename T>
@@ -242,115 +377,164 @@ __device__ void zero_local(const View<T>& w) {
   for (int q = threadIdx.x; q < n; q += blockDim.x) w.v[q] = (T)0;
 }
 
-// t = b - A v on the owned planes; t written at field index (global or local buffer).
-template <typename T>
-__device__ void residual(const View<T>& w, const T* b, bool b_local, int boff, T* t) {
-  const EngLevel<T>& L = *w.L;
-  const int n = (w.z1 - w.z0) * w.plane;
-  // two sites per iteration, both computed before either is stored, so that
-  // their loads overlap
-  auto value = [&](int q, int* gidx) {
-    int i, j, k;
-    split_xy(L, q, &i, &j, &k);
-    k += w.z0;
-    *gidx = (k * L.ny + j) * L.nx + i;
-    const T bb = b_local ? b[*gidx - boff] : ld_cg(b + *gidx);
-    return bb - stencil_row<T, true>(w, i, j, k);
-  };
-  for (int q = threadIdx.x; q < n; q += 2 * blockDim.x) {
-    const int q2 = q + blockDim.x;
-    int g1 = 0, g2 = 0;
-    const T r1 = value(q, &g1);
-    const T r2 = q2 < n ? value(q2, &g2) : (T)0;
-    t[g1] = r1;
-    if (q2 < n) t[g2] = r2;
+// t = b - A v on the owned planes; t written at field index (global or local
+// buffer).  A thread takes a column of the slab (one x, y) over a chunk of
+// planes: the x-y sums of a plane are formed once and kept for the five rows
+// that read them (9 shared loads per site instead of 45).
+template <typename T, bool D2>
+__device__ void residual_cols(const View<T>& w, const T* b, bool b_local, int boff, T* t) {
+  const LevReg<T> R(w);
+  const int cols = w.plane, np = w.z1 - w.z0;
+  if (np <= 0) return;
+  // chunks of planes: as many as give every thread one column
+  const int want = max(1, (int)blockDim.x / cols), kc = max((np + want - 1) / want, 1), chunks = (np + kc - 1) / kc;
+  for (int q = threadIdx.x; q < cols * chunks; q += blockDim.x) {
+    const int chunk = q / cols;
+    int i, j, dummy;
+    split_xy(*w.L, q - chunk * cols, &i, &j, &dummy);
+    const int k0 = chunk * kc, k1 = min(k0 + kc, np);
+    int c[9];
+    window_of<T, D2>(R, i, j, c);
+    T P1[5], P2[5];
+#pragma unroll
+    for (int d = 0; d < 4; ++d) plane_sums<T, D2, true>(R, R.v + (k0 - 2 + d) * R.pp, c, &P1[d], &P2[d]);
+    for (int k = k0; k < k1; ++k) {
+      plane_sums<T, D2, true>(R, R.v + (k + 2) * R.pp, c, &P1[4], &P2[4]);
+      const int gidx = ((k + R.z0) * R.ny + j) * R.nx + i;
+      const T bb = b_local ? b[gidx - boff] : ld_cg(b + gidx);
+      T row[12];
+      row_table(R.tab, k + R.z0, row);
+      T acc = (T)0;
+#pragma unroll
+      for (int d = 0; d < 5; ++d) acc += row[d] * P1[d] + row[5 + d] * P2[d];
+      t[gidx] = bb - acc;
+#pragma unroll
+      for (int d = 0; d < 4; ++d) {
+        P1[d] = P1[d + 1];
+        P2[d] = P2[d + 1];
+      }
+    }
   }
 }
 
-// b_c = P^T t on the coarse planes [Z0, Z1) of level Lc (tables on the fine level Lf).
 template <typename T>
-__device__ void restrict_to(const EngLevel<T>& Lf, const EngLevel<T>& Lc, const T* t, bool t_local, T* bc, int Z0,
-                            int Z1) {
-  const int n = (Z1 - Z0) * Lc.nx * Lc.ny;
+__device__ __forceinline__ void residual(const View<T>& w, const T* b, bool b_local, int boff, T* t) {
+  if (w.L->ny == 1)
+    residual_cols<T, true>(w, b, b_local, boff, t);
+  else
+    residual_cols<T, false>(w, b, b_local, boff, t);
+}
+
+// b_c = P^T t on the coarse planes [Z0, Z1) of level Lc (tables on the fine
+// level Lf).  All taps of a site are loaded before they are summed.
+template <typename T, bool D2>
+__device__ void restrict_taps(const EngLevel<T>& Lf, const EngLevel<T>& Lc, const T* t, bool t_local, T* bc, int Z0,
+                              int Z1) {
+  constexpr int NY = D2 ? 1 : 3;
+  const int nx = Lf.nx, ny = Lf.ny, ncx = Lc.nx, ncy = Lc.ny;
+  const int n = (Z1 - Z0) * ncx * ncy;
+  const int* rz_idx = Lf.rz_idx;
+  const T* rz_w = Lf.rz_w;
   for (int q = threadIdx.x; q < n; q += blockDim.x) {
     int I, J, K;
     split_xy(Lc, q, &I, &J, &K);
     K += Z0;
-    T acc = (T)0;
+    int col[NY * 3], kr[4];
+    T wz[4], x[4][NY * 3];
+#pragma unroll
+    for (int qy = 0; qy < NY; ++qy) {
+      const int row = D2 ? 0 : ewrap(2 * J + qy - 1, ny) * nx;
+#pragma unroll
+      for (int qx = 0; qx < 3; ++qx) col[qy * 3 + qx] = row + ewrap(2 * I + qx - 1, nx);
+    }
 #pragma unroll
     for (int qz = 0; qz < 4; ++qz) {
       // an unused tap (index -1) reads row 0 with weight 0: no branch between taps
-      const int kr = Lf.rz_idx[K * 4 + qz];
-      const int kf = kr < 0 ? 0 : kr;
-      const T wz = kr < 0 ? (T)0 : Lf.rz_w[K * 4 + qz];
-      for (int qy = -1; qy <= 1; ++qy) {
-        T wy;
-        int jf;
-        if (Lf.ny == 1) {
-          if (qy != 0) continue;
-          wy = (T)1;
-          jf = 0;
-        } else {
-          wy = qy == 0 ? (T)1 : (T)0.5;
-          jf = ewrap(2 * J + qy, Lf.ny);
-        }
+      kr[qz] = rz_idx[K * 4 + qz];
+      wz[qz] = kr[qz] < 0 ? (T)0 : rz_w[K * 4 + qz];
+      const T* tp = t + (kr[qz] < 0 ? 0 : kr[qz]) * ny * nx;
 #pragma unroll
-        for (int qx = -1; qx <= 1; ++qx) {
-          const T wx = qx == 0 ? (T)1 : (T)0.5;
-          const int idx = (kf * Lf.ny + jf) * Lf.nx + ewrap(2 * I + qx, Lf.nx);
-          acc += wz * wy * wx * (t_local ? t[idx] : ld_cg(t + idx));
-        }
-      }
-    }
-    bc[(K * Lc.ny + J) * Lc.nx + I] = acc;
-  }
-}
-
-// v_f += P v_c on the local planes [z0-2, z1+2) of the fine view (halo included).
-template <typename T>
-__device__ void prolong_into(const View<T>& w, const EngLevel<T>& Lc, const T* vc, bool vc_local, int vc_z0) {
-  const EngLevel<T>& L = *w.L;
-  const int p0 = max(0, w.z0 - 2), p1 = min(L.nz, w.z1 + 2);
-  const int n = (p1 - p0) * w.plane;
-  for (int q = threadIdx.x; q < n; q += blockDim.x) {
-    int i, j, k;
-    split_xy(L, q, &i, &j, &k);
-    k += p0;
-    int xi0 = i >> 1, xi1 = xi0;
-    T xw0 = (T)1, xw1 = (T)0;
-    if (i & 1) {
-      xi1 = ewrap(xi0 + 1, Lc.nx);
-      xw0 = xw1 = (T)0.5;
-    }
-    int yi0 = 0, yi1 = 0;
-    T yw0 = (T)1, yw1 = (T)0;
-    if (L.ny > 1) {
-      yi0 = yi1 = j >> 1;
-      if (j & 1) {
-        yi1 = ewrap(yi0 + 1, Lc.ny);
-        yw0 = yw1 = (T)0.5;
-      }
+      for (int c = 0; c < NY * 3; ++c) x[qz][c] = t_local ? tp[col[c]] : ld_cg(tp + col[c]);
     }
     T acc = (T)0;
 #pragma unroll
-    for (int qz = 0; qz < 2; ++qz) {
-      const int kr = L.pz_idx[k * 2 + qz];
-      const int kc = kr < 0 ? 0 : kr;
-      const T wz = kr < 0 ? (T)0 : L.pz_w[k * 2 + qz];
-      const int yi[2] = {yi0, yi1}, xi[2] = {xi0, xi1};
-      const T yw[2] = {yw0, yw1}, xw[2] = {xw0, xw1};
-      for (int a = 0; a < 2; ++a) {
-        if (yw[a] == (T)0) continue;
-        for (int c = 0; c < 2; ++c) {
-          if (xw[c] == (T)0) continue;
-          const int idx = vc_local ? ((kc - vc_z0 + 2) * Lc.pp + yi[a] * Lc.rp + xpos(xi[c], Lc.half))
-                                   : ((kc * Lc.ny + yi[a]) * Lc.nx + xi[c]);
-          acc += wz * yw[a] * xw[c] * (vc_local ? vc[idx] : ld_cg(vc + idx));
+    for (int qz = 0; qz < 4; ++qz)
+#pragma unroll
+      for (int qy = 0; qy < NY; ++qy) {
+        const T wy = D2 || qy == 1 ? (T)1 : (T)0.5;
+#pragma unroll
+        for (int qx = 0; qx < 3; ++qx) {
+          const T wx = qx == 1 ? (T)1 : (T)0.5;
+          acc += wz[qz] * wy * wx * x[qz][qy * 3 + qx];
         }
       }
-    }
-    w.v[w.loc(i, j, k)] += acc;
+    bc[(K * ncy + J) * ncx + I] = acc;
   }
+}
+
+template <typename T>
+__device__ __forceinline__ void restrict_to(const EngLevel<T>& Lf, const EngLevel<T>& Lc, const T* t, bool t_local,
+                                            T* bc, int Z0, int Z1) {
+  if (Lf.ny == 1)
+    restrict_taps<T, true>(Lf, Lc, t, t_local, bc, Z0, Z1);
+  else
+    restrict_taps<T, false>(Lf, Lc, t, t_local, bc, Z0, Z1);
+}
+
+// v_f += P v_c on the local planes [z0-2, z1+2) of the fine view (halo
+// included).  A thread takes the pair of fine sites 2 I, 2 I + 1 of a row: the
+// even one is the coarse node I in x, the odd one the mean of I and I + 1.
+template <typename T, bool D2>
+__device__ void prolong_pairs(const View<T>& w, const EngLevel<T>& Lc, const T* vc, bool vc_local, int vc_z0) {
+  const EngLevel<T>& L = *w.L;
+  const int nx = L.nx, ny = L.ny, rp = L.rp, pp = L.pp, half = L.half, z0 = w.z0;
+  const int ncx = Lc.nx, ncy = Lc.ny, crp = Lc.rp, cpp = Lc.pp, chalf = Lc.half;
+  const int* pz_idx = L.pz_idx;
+  const T* pz_w = L.pz_w;
+  const int p0 = max(0, z0 - 2), p1 = min(L.nz, w.z1 + 2);
+  const int hx = nx >> 1, n = (p1 - p0) * ny * hx;
+  const int lh = L.lx >= 1 ? L.lx - 1 : -1;
+  for (int q = threadIdx.x; q < n; q += blockDim.x) {
+    const int r = lh >= 0 ? q >> lh : q / hx;
+    const int I = lh >= 0 ? q & (hx - 1) : q - r * hx;
+    const int kr0 = D2 ? r : (L.ly >= 0 ? r >> L.ly : r / ny);
+    const int j = D2 ? 0 : (L.ly >= 0 ? r & (ny - 1) : r - kr0 * ny), k = p0 + kr0;
+    const int I1 = I + 1 == ncx ? 0 : I + 1;
+    const bool yo = !D2 && (j & 1) != 0;
+    const int yi[2] = {D2 ? 0 : j >> 1, yo ? ((j >> 1) + 1 == ncy ? 0 : (j >> 1) + 1) : 0};
+    const T yw = yo ? (T)0.5 : (T)1;
+    const int xa = vc_local ? xpos(I, chalf) : I, xb = vc_local ? xpos(I1, chalf) : I1;
+    T acc0 = (T)0, acc1 = (T)0;
+#pragma unroll
+    for (int qz = 0; qz < 2; ++qz) {
+      // an unused tap reads the row's first tap with weight 0
+      const int kr = pz_idx[k * 2 + qz];
+      const int kc = kr < 0 ? max(pz_idx[k * 2], 0) : kr;
+      const T wz = kr < 0 ? (T)0 : pz_w[k * 2 + qz];
+#pragma unroll
+      for (int a = 0; a < (D2 ? 1 : 2); ++a) {
+        if (a == 1 && !yo) continue;
+        const int row = vc_local ? (kc - vc_z0 + 2) * cpp + yi[a] * crp : (kc * ncy + yi[a]) * ncx;
+        const T u0 = vc_local ? vc[row + xa] : ld_cg(vc + row + xa);
+        const T u1 = vc_local ? vc[row + xb] : ld_cg(vc + row + xb);
+        acc0 += wz * yw * (T)1 * u0;
+        acc1 += wz * yw * (T)0.5 * u0;
+        acc1 += wz * yw * (T)0.5 * u1;
+      }
+    }
+    T* out = w.v + (k - z0 + 2) * pp + j * rp + I;
+    out[0] += acc0;
+    out[half] += acc1;
+  }
+}
+
+template <typename T>
+__device__ __forceinline__ void prolong_into(const View<T>& w, const EngLevel<T>& Lc, const T* vc, bool vc_local,
+                                             int vc_z0) {
+  if (w.L->ny == 1)
+    prolong_pairs<T, true>(w, Lc, vc, vc_local, vc_z0);
+  else
+    prolong_pairs<T, false>(w, Lc, vc, vc_local, vc_z0);
 }
 
 template <typename T>
@@ -424,17 +608,6 @@ __device__ void coarsest_step(const View<T>& w, int level, const T* b, double* y
   }
 }
 
-template <typename T, bool NOISE>
-__device__ void sweeps(const View<T>& w, int level, int first_sweep, int count, const T* b, bool b_local, int boff, Key key,
-                       unsigned long long cyc, int rank, int csize, bool cluster) {
-  const Sync sync{cluster};
-  for (int s = 0; s < count; ++s)
-    for (int q = 0; q < w.L->ncol; ++q) {
-      colour_pass<T, NOISE>(w, level, q, first_sweep + s, b, b_local, boff, key, cyc, rank, csize, cluster);
-      sync();
-    }
-}
-
 // Fills the colour-class table of the staged level L as seen by the CTA
 // owning planes [z0, z1): per class the geometry and the owned rank range.
 // (No barrier: the caller syncs.)
@@ -458,7 +631,54 @@ __device__ void stage_colours(const EngLevel<T>& L, int z0, int z1, EngColour* c
     const int pr = c.nxc * c.nyc;
     c.rank_lo = kk_lo * pr;
     c.nsite = (c.nxc > 0 && c.nyc > 0 && nzc > 0 && kk_hi > kk_lo) ? (kk_hi - kk_lo) * pr : 0;
+    c.noff = 0;
     col[q] = c;
+  }
+}
+
+// The normals of every sweep of the levels that the plan gave a buffer, drawn
+// once at the start of the launch by all threads, a whole Philox block at a
+// time: a cluster level's by the CTA that owns the planes, CTA 0's levels by
+// all CTAs of the cluster (through distributed shared memory).  The cluster
+// barrier before the first use orders them.  Normal of (sweep, class, rank)
+// at [sweep * sites per CTA + the class's offset + rank - its first rank].
+template <typename T>
+__device__ void stage_noise(const EngParams<T>* P, const EngRun& run, unsigned char* smem, const EngLevel<T>* lev0,
+                            const EngColour* col0, int rank, int csize, unsigned long long cyc) {
+  const int lt = P->l0, lc = P->L - 1, ns = run.mu1 + run.mu2;
+  for (int l = lt; l <= lc; ++l) {
+    if (P->nz_off[l] < 0 || (l == lc && run.coarse_mode == SELM_COARSE_CHOLESKY)) continue;
+    const EngLevel<T>& L = lev0[l - lt];
+    const EngColour* col = col0 + (size_t)(l - lt) * kEngMaxColours;
+    const bool own = L.cluster != 0;
+    T* dst = reinterpret_cast<T*>(smem + P->nz_off[l]);
+    if (!own && csize > 1) dst = cg::this_cluster().map_shared_rank(dst, 0);
+    const int stride = L.P * L.nx * L.ny, ncol = L.ncol;
+    int gmax = 0;   // noise groups of the largest class
+    for (int q = 0; q < ncol; ++q)
+      if (col[q].nsite > 0) gmax = max(gmax, ((col[q].rank_lo + col[q].nsite - 1) >> 2) - (col[q].rank_lo >> 2) + 1);
+    const int total = ns * ncol * gmax;
+    const int first = own ? threadIdx.x : rank * blockDim.x + threadIdx.x;
+    const int step = own ? blockDim.x : csize * blockDim.x;
+    for (int t = first; t < total; t += step) {
+      const int u = t / gmax, sweep = u / ncol, q = u - sweep * ncol;
+      const EngColour& c = col[q];
+      const int g = (c.rank_lo >> 2) + t - u * gmax;
+      if (c.nsite <= 0 || 4 * g >= c.rank_lo + c.nsite) continue;
+      T n4[4];
+      Normals<T>::get(eng_philox10(make_uint4((uint32_t)g,
+                                              (uint32_t)l | ((uint32_t)L.comp_id << 4) | ((uint32_t)q << 8) |
+                                                  ((uint32_t)sweep << 12),
+                                              (uint32_t)cyc, (uint32_t)(cyc >> 32)),
+                                   run.key.k0, run.key.k1),
+                      n4);
+      T* out = dst + (size_t)sweep * stride + c.noff;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int s = 4 * g + e - c.rank_lo;
+        if (s >= 0 && s < c.nsite) out[s] = n4[e];
+      }
+    }
   }
 }
 
@@ -558,6 +778,14 @@ __global__ void __launch_bounds__(EngThreads<T>::value, 1) k_coarse_engine(const
       }
     }
     __syncthreads();
+    if (threadIdx.x >= 32 && threadIdx.x <= 32 + lc - lt) {   // offset of each class in the level's normals
+      const int l = lt + threadIdx.x - 32;
+      int off = 0;
+      for (int q = 0; q < sl_at(l).ncol; ++q) {
+        col_at(l)[q].noff = off;
+        off += col_at(l)[q].nsite;
+      }
+    }
     if (threadIdx.x == 0)
       for (int l = lt; l < lc; ++l) {
         EngLevel<T>& L = sl_at(l);
@@ -576,7 +804,26 @@ __global__ void __launch_bounds__(EngThreads<T>::value, 1) k_coarse_engine(const
     w.col = col_at(l);
     return w;
   };
+  if (NOISE) stage_noise<T>(P, run, smem, lev0, col0, rank, csize, cyc);
+  // the sweeps of level l from sweep index `first`, with b in shared memory
+  // (blocal) or read from L2
+  auto pass_args = [&](int l, int first, const T* b, bool blocal, int boff) {
+    const EngLevel<T>& L = sl_at(l);
+    PassArgs<T> A;
+    A.level = l;
+    A.first = first;
+    A.b = b;
+    A.b_local = blocal;
+    A.boff = boff;
+    A.noise = NOISE && P->nz_off[l] >= 0 ? reinterpret_cast<const T*>(smem + P->nz_off[l]) : nullptr;
+    A.nstride = L.P * L.nx * L.ny;
+    A.c1 = (uint32_t)l | ((uint32_t)L.comp_id << 4);
+    A.key = key;
+    A.cyc = cyc;
+    return A;
+  };
 
+  pdl_wait();   // everything above reads only the plan and the counter
   // ---- down leg over the cluster levels ----
   int l = lt;
   for (; l < lc && sl_at(l).cluster; ++l) {
@@ -590,7 +837,7 @@ __global__ void __launch_bounds__(EngThreads<T>::value, 1) k_coarse_engine(const
     const int boff = bl ? w.z0 * w.plane : 0;
     if (bl) load_owned(w, L.gb, (T*)(smem + L.sb));
     cl.sync();
-    sweeps<T, NOISE>(w, l, 0, mu1, bsrc, bl, boff, key, cyc, rank, csize, true);
+    sweeps_any<T, NOISE>(w, pass_args(l, 0, bsrc, bl, boff), mu1, rank, csize, true);
     residual(w, bsrc, bl, boff, L.gt);
     cl.sync();
     // the coarse planes of the restriction are split over the cluster's CTAs
@@ -604,6 +851,11 @@ __global__ void __launch_bounds__(EngThreads<T>::value, 1) k_coarse_engine(const
     cl.sync();
   }
   const int lsingle = l;   // first level held by CTA 0 alone
+  if (lsingle == lt && csize > 1) {
+    // no cluster level: the other CTAs were here for the normals only
+    cl.sync();
+    if (rank != 0) return;
+  }
   if (rank == 0) {
     // ---- single-CTA part: levels lsingle .. lc and back ----
     if (lsingle == lt) {   // b from global only when no cluster level restricted into it
@@ -621,9 +873,9 @@ __global__ void __launch_bounds__(EngThreads<T>::value, 1) k_coarse_engine(const
         __syncthreads();
         break;
       }
-      sweeps<T, NOISE>(w, k, 0, mu1, b, true, 0, key, cyc, 0, 1, false);
+      sweeps_any<T, NOISE>(w, pass_args(k, 0, b, true, 0), mu1, 0, 1, false);
       if (k == lc) {
-        sweeps<T, NOISE>(w, k, mu1, mu2, b, true, 0, key, cyc, 0, 1, false);
+        sweeps_any<T, NOISE>(w, pass_args(k, mu1, b, true, 0), mu2, 0, 1, false);
         break;
       }
       const EngLevel<T>& Lc = sl_at(k + 1);
@@ -638,13 +890,14 @@ __global__ void __launch_bounds__(EngThreads<T>::value, 1) k_coarse_engine(const
       View<T> w = view_of(k, false);
       prolong_into(w, Lc, (const T*)(smem + Lc.sv), true, 0);
       __syncthreads();
-      sweeps<T, NOISE>(w, k, mu1, mu2, (const T*)(smem + L.sb), true, 0, key, cyc, 0, 1, false);
+      sweeps_any<T, NOISE>(w, pass_args(k, mu1, (const T*)(smem + L.sb), true, 0), mu2, 0, 1, false);
     }
     {   // the engine's result, or the hand-off to the cluster's prolongation
       View<T> w = view_of(lsingle, false);
       store_owned(w, sl_at(lsingle).gv);
     }
   }
+  if (lsingle == lt) return;
   cl.sync();
   // ---- up leg over the cluster levels ----
   for (int k = lsingle - 1; k >= lt; --k) {
@@ -655,16 +908,26 @@ __global__ void __launch_bounds__(EngThreads<T>::value, 1) k_coarse_engine(const
       prolong_into(w, Lc, Lc.gv, false, 0);
     } else {
       // the coarse level is held by CTA 0, which still has its v in shared
-      // memory; the other CTAs first copy it (independent loads) into their own
-      // unused slab of that level, then prolong from shared memory
+      // memory; the other CTAs first copy the coarse planes that their slab and
+      // halo read (independent loads) into their own unused slab of that
+      // level, then prolong from shared memory
       View<T> wc = view_of(k + 1, false);
       if (rank != 0) {
-        const int nc = Lc.nx * Lc.ny * Lc.nz;
+        const int p0 = max(0, w.z0 - 2), p1 = min(L.nz, w.z1 + 2);
+        int c0 = Lc.nz, c1 = 0;
+        for (int z = p0; z < p1; ++z)
+#pragma unroll
+          for (int t = 0; t < 2; ++t) {
+            const int kr = L.pz_idx[2 * z + t], kc = kr < 0 ? max(L.pz_idx[2 * z], 0) : kr;
+            c0 = min(c0, kc);
+            c1 = max(c1, kc + 1);
+          }
+        const int base = c0 * wc.plane, nc = max(0, c1 - c0) * wc.plane;
 #pragma unroll 4
         for (int q = threadIdx.x; q < nc; q += blockDim.x) {
           int i, j, kk;
           split_xy(Lc, q, &i, &j, &kk);
-          wc.v[wc.loc(i, j, kk)] = ld_cg(Lc.gv + q);
+          wc.v[wc.loc(i, j, c0 + kk)] = ld_cg(Lc.gv + base + q);
         }
         __syncthreads();
       }
@@ -672,8 +935,8 @@ __global__ void __launch_bounds__(EngThreads<T>::value, 1) k_coarse_engine(const
     }
     cl.sync();
     const bool bl = L.sb >= 0;   // staged on the way down, untouched since
-    sweeps<T, NOISE>(w, k, mu1, mu2, bl ? (const T*)(smem + L.sb) : L.gb, bl, bl ? w.z0 * w.plane : 0, key, cyc, rank,
-                     csize, true);
+    sweeps_any<T, NOISE>(w, pass_args(k, mu1, bl ? (const T*)(smem + L.sb) : L.gb, bl, bl ? w.z0 * w.plane : 0), mu2,
+                         rank, csize, true);
     store_owned(w, L.gv);
     cl.sync();
   }
@@ -717,7 +980,7 @@ void slab_pitches(int nx, int ny, int mz, int* half, int* rp, int* pp) {
 }
 
 template <typename T>
-bool try_plan(const LevelDev* levs, int L, int l0, int C, bool stage_b, size_t smem_cap, EnginePlanT<T>* out) {
+bool try_plan(const LevelDev* levs, int L, int l0, int C, bool stage_b, int sweeps, size_t smem_cap, EnginePlanT<T>* out) {
   // cluster levels first (largest), then single levels
   const int ncomp = levs[0].ncomp;
   size_t need_max = 0;
@@ -814,6 +1077,22 @@ bool try_plan(const LevelDev* levs, int L, int l0, int C, bool stage_b, size_t s
   p.xfw_off = (int)xfw_off;
   out->smem_bytes = align16(xfw_off + (size_t)xrows * sizeof(T));
   if (out->smem_bytes > smem_cap) return false;
+  // normals of the noisy launches, in what is left: the coarsest levels first
+  // (their passes are the shortest); a level without room draws at its sites
+  out->smem_noise = out->smem_bytes;
+  for (int l = 0; l < kMaxLevels; ++l) p.nz_off[l] = -1;
+  for (int l = L - 1; l >= l0; --l) {
+    size_t sites = 0;
+    for (int c = 0; c < ncomp; ++c) {
+      const CompDev& d = levs[l].c[c];
+      const size_t n = (size_t)p.comp[c].lev[l].P * d.nx * d.ny;
+      sites = sites > n ? sites : n;
+    }
+    const size_t bytes = align16(sites * (size_t)sweeps * sizeof(T));
+    if (out->smem_noise + bytes > smem_cap) break;
+    p.nz_off[l] = (int)out->smem_noise;
+    out->smem_noise += bytes;
+  }
   out->cluster = C;
   return true;
 }
@@ -890,7 +1169,7 @@ bool raise_smem_limit() {
 
 template <typename T>
 bool plan_coarse_engine(const LevelDev* levs, int L, void* const* gb, void* const* gv, void* const* gt,
-                        void* dev_params, cudaStream_t st, EnginePlanT<T>* plan, int want_cluster,
+                        void* dev_params, cudaStream_t st, EnginePlanT<T>* plan, int sweeps, int want_cluster,
                         int min_level) {
   static_assert(sizeof(EngParams<T>) <= kEngParamBytes, "engine plan exceeds its workspace slot");
   plan->valid = false;
@@ -909,32 +1188,42 @@ bool plan_coarse_engine(const LevelDev* levs, int L, void* const* gb, void* cons
       if (want_cluster > 0 && C > want_cluster) continue;
       EnginePlanT<T> cand{};
       // with b of the cluster levels staged in shared memory if it fits
-      if (!try_plan<T>(levs, L, l0, C, true, smem_cap, &cand) &&
-          !try_plan<T>(levs, L, l0, C, false, smem_cap, &cand))
+      if (!try_plan<T>(levs, L, l0, C, true, sweeps, smem_cap, &cand) &&
+          !try_plan<T>(levs, L, l0, C, false, sweeps, smem_cap, &cand))
         continue;
       // The dynamic shared-memory limit is a per-kernel setting shared by every
       // handle of the process: raise it once to the device maximum so that
       // plans of any size stay launchable.
       if (!raise_smem_limit<T>()) continue;
-      if (cand.cluster > 1) {
-        auto fn = k_coarse_engine<T, true>;
+      auto fits = [&](int c, size_t smem) {
         cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3(cand.cluster * levs[0].ncomp);
+        cfg.gridDim = dim3(c * levs[0].ncomp);
         cfg.blockDim = dim3(EngThreads<T>::value);
-        cfg.dynamicSmemBytes = cand.smem_bytes;
+        cfg.dynamicSmemBytes = smem;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = cand.cluster;
+        attr[0].val.clusterDim.x = c;
         attr[0].val.clusterDim.y = 1;
         attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int nclusters = 0;
-        if (cudaOccupancyMaxActiveClusters(&nclusters, fn, &cfg) != cudaSuccess || nclusters < 1) {
-          cudaGetLastError();
-          continue;
+        if (cudaOccupancyMaxActiveClusters(&nclusters, k_coarse_engine<T, true>, &cfg) == cudaSuccess && nclusters >= 1)
+          return true;
+        cudaGetLastError();
+        return false;
+      };
+      if (cand.cluster > 1 && !fits(cand.cluster, cand.smem_noise)) continue;
+      // Without cluster levels CTA 0 holds everything; the noisy launch takes
+      // more CTAs to draw its normals (FP64 Box-Muller at two lanes per clock
+      // is most of such a cycle on one SM).
+      cand.noise_cluster = cand.cluster;
+      for (int c = 16; cand.cluster == 1 && c > 1; c /= 2)
+        if (cluster_ok && (want_cluster <= 0 || c <= want_cluster) && cand.params.nz_off[l0] >= 0 &&
+            fits(c, cand.smem_noise)) {
+          cand.noise_cluster = c;
+          break;
         }
-      }
       *plan = cand;
       fill_engine_tables<T>(levs, L, gb, gv, gt, plan);
       if (cudaMemcpyAsync(dev_params, &plan->params, sizeof(EngParams<T>), cudaMemcpyHostToDevice, st) !=
@@ -955,27 +1244,32 @@ template <typename T>
 cudaError_t launch_coarse_engine(const EnginePlanT<T>& plan, int mu1, int mu2, int coarse_mode, bool noise, Key key,
                                  const unsigned long long* cyc, cudaStream_t st) {
   EngRun run{mu1, mu2, coarse_mode, key, cyc};
+  const int cluster = noise ? plan.noise_cluster : plan.cluster;
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(plan.cluster * plan.params.ncomp);
+  cfg.gridDim = dim3(cluster * plan.params.ncomp);
   cfg.blockDim = dim3(EngThreads<T>::value);
-  cfg.dynamicSmemBytes = plan.smem_bytes;
+  cfg.dynamicSmemBytes = noise ? plan.smem_noise : plan.smem_bytes;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  // Programmatic launch: the tables and normals are staged while the kernel
+  // before it drains.
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = plan.cluster;
+  attr[0].val.clusterDim.x = cluster;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   prof::Scope ps(SELM_K_COARSE_SWEEP, st);
   if (noise) return cudaLaunchKernelEx(&cfg, k_coarse_engine<T, true>, plan.dev, run);
   return cudaLaunchKernelEx(&cfg, k_coarse_engine<T, false>, plan.dev, run);
 }
 
 template bool plan_coarse_engine<float>(const LevelDev*, int, void* const*, void* const*, void* const*, void*,
-                                        cudaStream_t, EnginePlanT<float>*, int, int);
+                                        cudaStream_t, EnginePlanT<float>*, int, int, int);
 template bool plan_coarse_engine<double>(const LevelDev*, int, void* const*, void* const*, void* const*, void*,
-                                         cudaStream_t, EnginePlanT<double>*, int, int);
+                                         cudaStream_t, EnginePlanT<double>*, int, int, int);
 template cudaError_t launch_coarse_engine<float>(const EnginePlanT<float>&, int, int, int, bool, Key,
                                                  const unsigned long long*, cudaStream_t);
 template cudaError_t launch_coarse_engine<double>(const EnginePlanT<double>&, int, int, int, bool, Key,

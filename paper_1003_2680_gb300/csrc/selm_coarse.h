@@ -46,6 +46,7 @@ struct EngColour {
   int rank_lo, nsite;   // ranks of the class owned by this CTA: [rank_lo, rank_lo + nsite)
   float inv_nxc, inv_nyc;
   int sx, sy;           // log2 of nxc / nyc when they are powers of two, else -1
+  int noff;             // owned sites of the classes before it (offset into a sweep's normals)
 };
 
 constexpr int kEngMaxColours = 16;
@@ -74,6 +75,7 @@ struct EngParams {
   // at [2 nz_l + 4K, 2 nz_l + 4K + 4).
   int xfi_off, xfw_off;
   int xf_row[kMaxLevels];
+  int nz_off[kMaxLevels];   // normals of the level's sweeps (byte offset), -1: drawn at the sites
   EngComp<T> comp[kMaxComps];
 };
 
@@ -88,7 +90,9 @@ template <typename T>
 struct EnginePlanT {
   bool valid = false;
   int cluster = 1;
-  size_t smem_bytes = 0;
+  size_t smem_bytes = 0;      // noise-free launches
+  size_t smem_noise = 0;      // with the buffers of normals
+  int noise_cluster = 1;      // cluster of the noisy launches (helpers that only draw, without cluster levels)
   size_t y_off_comp[kMaxComps] = {};
   EngParams<T> params{};
   const EngParams<T>* dev = nullptr;   // device copy of params
@@ -101,10 +105,11 @@ constexpr size_t kEngParamBytes = 32768;
 // first level whose slabs fit in shared memory).  gb/gv/gt: per-level global
 // field pointers.  dev_params: kEngParamBytes of device memory that receives
 // the plan (copied on `st`, which is synchronised before returning).
+// sweeps: mu1 + mu2 of the launches (sizes the buffers of normals).
 // want_cluster > 0 caps the cluster size (the autotuner's knob).
 template <typename T>
 bool plan_coarse_engine(const LevelDev* levs, int L, void* const* gb, void* const* gv, void* const* gt,
-                        void* dev_params, cudaStream_t st, EnginePlanT<T>* plan, int want_cluster = 0,
+                        void* dev_params, cudaStream_t st, EnginePlanT<T>* plan, int sweeps, int want_cluster = 0,
                         int min_level = 1);
 
 // Runs the V-cycle below level l0-1: reads b at level l0, writes v at level l0.

@@ -1,0 +1,36 @@
+"""The coarse engine where its slabs, classes and buffers of normals come out
+uneven: odd class extents, a last slab with fewer planes, normals that do not
+fit beside the level (96^3 in FP32), CTA 0 alone with helpers drawing for it
+(2-D in FP64).  One stochastic V-cycle against the oracle at the parity tests'
+field tolerances (1e-12 in FP64, 1e-5 in FP32)."""
+
+import pytest
+import torch
+
+import selm_inputs
+from oracle import grid, multigrid, philox
+from tests.gpu_util import from_dev, rel, round_like, to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("dim,n,prec,mode", [(3, 40, "fp32", 0), (3, 40, "fp64", 0), (3, 72, "fp32", 0),
+                                             (3, 96, "fp32", 0), (2, 96, "fp64", 0), (2, 160, "fp32", 0),
+                                             (3, 24, "fp32", 1), (2, 48, "fp64", 1)])
+def test_uneven_vcycle(dim, n, prec, mode):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1003_2680_gb300 import selm as S
+    dt, tol = (torch.float64, 1e-12) if prec == "fp64" else (torch.float32, 1e-5)
+    m = S.SelmMG(dim=dim, n=n, levels=3 if mode else 0, precision=0 if prec == "fp64" else 1, coarse_mode=mode,
+                 seed=11, instance=3)
+    assert S.selm_mg_engine_info(m.h)[0] >= 1
+    osys = grid.velocity_system(n, dim, levels=S.selm_mg_levels(m.h))
+    v0 = round_like(selm_inputs.fields(osys.shapes(0), seed=1), dt)
+    b0 = round_like(selm_inputs.fields(osys.shapes(0), seed=2), dt)
+    v, b = to_dev(m.h, v0, dt), to_dev(m.h, b0, dt)
+    S.selm_mg_vcycle(m.h, 0, v, b, 7, 1)
+    want = [x.copy() for x in v0]
+    multigrid.vcycle(osys, 0, want, b0, philox.PhiloxNoise(11, 3, 7), 1.0,
+                     coarse_mode="smooth" if mode else "cholesky")
+    assert rel(from_dev(m.h, v), want) < tol
