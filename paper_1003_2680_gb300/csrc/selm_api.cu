@@ -253,6 +253,18 @@ void bind_system(Sys* s, int si, const Plan& p, char* ws, int fsi = -1) {
 
 inline cudaStream_t S(void* st) { return (cudaStream_t)st; }
 
+long long level_sites(const LevelDev& L) {   // of the largest component
+  long long big = 0;
+  for (int c = 0; c < L.ncomp; ++c) {
+    const long long n = (long long)L.c[c].nx * L.c[c].ny * L.c[c].nz;
+    big = n > big ? n : big;
+  }
+  return big;
+}
+
+// Levels of at most 2^20 sites per component may run as cooperative launches.
+constexpr long long kCoopMaxSites = 1ll << 20;
+
 Sys* sys_of(selm_mg* h, int system) {
   if (system == SELM_SYS_VELOCITY) return &h->vel;
   if (system == SELM_SYS_PRESSURE && h->has_pres) return &h->pres;
@@ -276,10 +288,7 @@ selm_status vcycle_t(selm_mg* h, Sys& s, int l, T* v0, const T* b0, bool noise, 
   // of its V-cycle in one cooperative launch (one or a few site updates per
   // thread per pass).  Larger levels keep one GPU-wide launch per colour pass,
   // whose parallelism then beats the launch overhead.
-  bool coop_size = true;
-  for (int c = 0; c < L.ncomp; ++c)
-    if ((long long)L.c[c].nx * L.c[c].ny * L.c[c].nz > (1ll << 20)) coop_size = false;
-  if (l > 0 && !last && !L.rb && coop_size && s.use_engine && s.use_coop && eng.valid && l < eng.params.l0 &&
+  if (l > 0 && !last && !L.rb && level_sites(L) <= kCoopMaxSites && s.use_engine && s.use_coop && eng.valid && l < eng.params.l0 &&
       s.coop_bar && level_coop_supported<T>(L)) {
     const LevelDev& Lc = s.lev[l + 1];
     CK(launch_level_coop<T>(L, Lc, 0, h->mu1, h->mu2, v, b, (T*)s.t[l], (T*)s.b[l + 1], (T*)s.v[l + 1], s.coop_bar,
@@ -592,18 +601,19 @@ namespace {
 // then spreads over every SM instead of one cluster per component, which
 // pays once a component holds 2^17 sites or more) and the engine starts at
 // level 2; otherwise the engine takes every level from 1.
+// FP64: the FP64 pipe bounds a pass, so levels of more than 2^15 sites stay
+// with the cooperative launches (a pass of a 40^3 level: about 12 us in a
+// cluster, 6 us over the GPU; of a 20^3 level: 3.4 and 5 us).
 int engine_first_level(const selm_mg* h, const Sys& s) {
-  if (s.engine_level > 0) return s.engine_level;
-  if (!s.use_coop || s.levels < 4) return 1;
-  long long big = 0;
-  for (int c = 0; c < s.lev[1].ncomp; ++c) {
-    const CompDev& d = s.lev[1].c[c];
-    const long long n = (long long)d.nx * d.ny * d.nz;
-    big = n > big ? n : big;
-  }
-  if (big < (1ll << 17)) return 1;
-  const bool ok = h->esize == 4 ? level_coop_supported<float>(s.lev[1]) : level_coop_supported<double>(s.lev[1]);
-  return ok ? 2 : 1;
+  auto coop = [&](int l) {
+    return h->esize == 4 ? level_coop_supported<float>(s.lev[l]) : level_coop_supported<double>(s.lev[l]);
+  };
+  int first = s.engine_level > 0 ? s.engine_level : 1;
+  if (s.engine_level <= 0 && s.use_coop && s.levels >= 4 && level_sites(s.lev[1]) >= (1ll << 17) && coop(1)) first = 2;
+  while (h->esize == 8 && s.use_coop && first + 2 < s.levels && !s.lev[first].rb &&
+         level_sites(s.lev[first]) > (1ll << 15) && level_sites(s.lev[first]) <= kCoopMaxSites && coop(first))
+    ++first;
+  return first;
 }
 
 }  // namespace

@@ -21,18 +21,23 @@
 //
 // What bounds it: latency.  A pass is a barrier, a site's 45 shared loads and
 // its sum, and about 150 passes follow one another.  So a level's constants
-// sit in registers, everything about a site but the values v is loaded before
-// the barrier that releases its pass, and the normals of a noisy launch are
-// drawn once at its start.  64^3 velocity V-cycle (levels of 32^3 and below),
-// one launch: 157 -> 128 us, noisy 211 -> 174 us; a pass of the 32^3 level 1.15
-// -> 0.81 us; residual of the 16^3 level in CTA 0 9.9 -> 3.1 us, prolongation
-// from it 9.8 -> 4.1 us.
+// sit in registers, all of a site's loads are issued before the first sum,
+// everything about a site but the values v is loaded off the critical path,
+// the normals of a noisy launch are drawn once at its start, and the coarsest
+// step is spread over the cluster.  64^3 velocity V-cycle (levels of 32^3 and
+// below), one launch: 157 -> 121 us, noisy 211 -> 150 us; 48^3: 125 -> 90,
+// noisy 184 -> 107 us; 96^3: 235 -> 204, noisy 353 -> 272 us.  Where the 121 us
+// go: 48 passes of 32^3 at 0.8 us, of 16^3 at 0.7 us, of 8^3 at 0.3 us, the
+// coarsest step 5 us, transfers 17 us, staging 5 us.
+// The 2-D and 3-D forms are separate kernels: as branches of one kernel their
+// code, twice as long, came from L2 anew in every launch (138 instead of 121 us).
 
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <atomic>
 #include <cstdint>
+#include <type_traits>
 
 #include "../../include/selm_mg.h"
 #include "selm_coarse.h"
@@ -46,14 +51,13 @@ namespace cg = cooperative_groups;
 namespace selm {
 namespace {
 
-// Threads per CTA.  FP32: 512, which leaves up to 128 registers a thread for
-// the unrolled 45-point row (at 1024 threads the 64-register cap spills it and
-// the colour passes on the engine's levels run slower).  FP64: 256; a row
-// takes twice the registers, and the FP64 pipe (two lanes per clock) is busy
-// with eight warps.
+// Threads per CTA.  FP32: 384, so that a thread has 168 registers for the 45
+// loads of a row in flight at once (512 threads: 128 registers, spills; a pass
+// of an 8^3 level 0.37 instead of 0.31 us).  FP64: 256; a row takes twice the
+// registers, and the FP64 pipe (two lanes per clock) is busy with eight warps.
 template <typename T>
 struct EngThreads {
-  static constexpr int value = sizeof(T) == 4 ? 512 : 256;
+  static constexpr int value = sizeof(T) == 4 ? 384 : 256;
 };
 
 __device__ __forceinline__ uint4 eng_philox10(uint4 c, uint32_t k0, uint32_t k1) { return philox4x32_10(c, k0, k1); }
@@ -129,29 +133,39 @@ __device__ __forceinline__ int fdiv(int n, int d, float inv) {
   return q;
 }
 
+// The launch's dynamic shared memory.  What the passes read is addressed by
+// element numbers from here (32-bit shared-memory addressing).
+template <typename T>
+__device__ __forceinline__ T* sm() {
+  extern __shared__ __align__(16) unsigned char smem[];
+  return reinterpret_cast<T*>(smem);
+}
+template <typename T>
+__device__ __forceinline__ int sm_at(const T* p) {
+  return (int)(p - sm<T>());
+}
+
 // A level's constants in registers: the passes read them at every site, and
 // the compiler cannot keep shared-memory values across the stores of v.
 template <typename T>
 struct LevReg {
   int nx, ny, mx, my, mz, half, rp, pp, z0, ncol, P;
   int xlast;        // position of x = nx - 1 in a row
-  T* v;             // plane z0 of the slab
-  const T* tab;
-  const EngColour* col;
-  T w1[9], w2[9];
+  int v;            // plane z0 of the slab (element of sm<T>())
+  int tab;          // row tables
+  int col;          // colour classes (byte of sm)
+  // w1 and w2 at a corner, a y edge, an x edge and the centre of the 3 x 3 window
+  T a0, a1, a3, a4, b0, b1, b3, b4;
   __device__ __forceinline__ explicit LevReg(const View<T>& w) {
     const EngLevel<T>& L = *w.L;
     nx = L.nx; ny = L.ny; mx = L.mx; my = L.my; mz = L.mz;
     half = L.half; rp = L.rp; pp = L.pp; z0 = w.z0; ncol = L.ncol; P = L.P;
     xlast = xpos(L.nx - 1, L.half);
-    v = w.v + 2 * pp;
-    tab = w.tab;
-    col = w.col;
-#pragma unroll
-    for (int q = 0; q < 9; ++q) {
-      w1[q] = L.w1[q];
-      w2[q] = L.w2[q];
-    }
+    v = sm_at(w.v) + 2 * pp;
+    tab = sm_at(w.tab);
+    col = (int)(reinterpret_cast<const unsigned char*>(w.col) - sm<unsigned char>());
+    a0 = L.w1[0]; a1 = L.w1[1]; a3 = L.w1[3]; a4 = L.w1[4];
+    b0 = L.w2[0]; b1 = L.w2[1]; b3 = L.w2[3]; b4 = L.w2[4];
   }
 };
 
@@ -175,25 +189,26 @@ __device__ __forceinline__ void window_of(const LevReg<T>& R, int i, int j, int 
 // The two x-y partial sums w1 . v and w2 . v of one plane (separable form of
 // the Galerkin row); CENTRE == false leaves out the site itself.
 template <typename T, bool D2, bool CENTRE>
-__device__ __forceinline__ void plane_sums(const LevReg<T>& R, const T* vp, const int c[9], T* s1, T* s2) {
+__device__ __forceinline__ void plane_sums(const LevReg<T>& R, int plane, const int c[9], T* s1, T* s2) {
+  const T* vp = sm<T>() + plane;
   T p1, p2;
   if (D2) {
     const T a = vp[c[3]], d = vp[c[5]];
-    p1 = R.w1[3] * a + R.w1[5] * d;
-    p2 = R.w2[3] * a + R.w2[5] * d;
+    p1 = R.a3 * a + R.a3 * d;
+    p2 = R.b3 * a + R.b3 * d;
   } else {
     const T a0 = vp[c[0]], b0 = vp[c[1]], c0 = vp[c[2]];
     const T a1 = vp[c[3]], c1 = vp[c[5]];
     const T a2 = vp[c[6]], b2 = vp[c[7]], c2 = vp[c[8]];
-    p1 = R.w1[0] * a0 + R.w1[1] * b0 + R.w1[2] * c0 + R.w1[3] * a1 + R.w1[5] * c1 + R.w1[6] * a2 + R.w1[7] * b2 +
-         R.w1[8] * c2;
-    p2 = R.w2[0] * a0 + R.w2[1] * b0 + R.w2[2] * c0 + R.w2[3] * a1 + R.w2[5] * c1 + R.w2[6] * a2 + R.w2[7] * b2 +
-         R.w2[8] * c2;
+    p1 = R.a0 * a0 + R.a1 * b0 + R.a0 * c0 + R.a3 * a1 + R.a3 * c1 + R.a0 * a2 + R.a1 * b2 +
+         R.a0 * c2;
+    p2 = R.b0 * a0 + R.b1 * b0 + R.b0 * c0 + R.b3 * a1 + R.b3 * c1 + R.b0 * a2 + R.b1 * b2 +
+         R.b0 * c2;
   }
   if (CENTRE) {
     const T b1 = vp[c[4]];
-    p1 += R.w1[4] * b1;
-    p2 += R.w2[4] * b1;
+    p1 += R.a4 * b1;
+    p2 += R.b4 * b1;
   }
   *s1 = p1;
   *s2 = p2;
@@ -229,10 +244,10 @@ struct Site {
 template <typename T>
 struct PassArgs {
   int level, first;            // sweep index of the first pass
-  const T* b;
+  const T* gb;                 // b of the level in global memory, or
+  int sb;                      // the owned planes' b (element of sm<T>(), less the first plane's field index)
   bool b_local;
-  int boff;
-  const T* noise;              // normals of every sweep, or null: formed here
+  int noise;                   // normals of every sweep (element of sm<T>()), -1: formed here
   int nstride;                 // normals per sweep
   uint32_t c1;                 // level and component of the noise counter
   Key key;
@@ -263,10 +278,10 @@ __device__ __forceinline__ void load_site(const LevReg<T>& R, const PassArgs<T>&
   const int i = cc.cx + R.mx * ii, j = cc.cy + R.my * jj, k = cc.cz + R.mz * kk;
   x.kz = k - R.z0;
   const int gidx = (k * R.ny + j) * R.nx + i;
-  x.b = A.b_local ? A.b[gidx - A.boff] : ld_cg(A.b + gidx);
+  x.b = A.b_local ? sm<T>()[A.sb + gidx] : ld_cg(A.gb + gidx);
   if (NOISE) {
-    if (A.noise) {
-      x.n = A.noise[sweep * A.nstride + cc.noff + s];
+    if (A.noise >= 0) {
+      x.n = sm<T>()[A.noise + sweep * A.nstride + cc.noff + s];
     } else {
       normal_of(eng_philox10(make_uint4((uint32_t)(rk >> 2), A.c1 | ((uint32_t)q << 8) | ((uint32_t)sweep << 12),
                                         (uint32_t)A.cyc, (uint32_t)(A.cyc >> 32)),
@@ -275,26 +290,95 @@ __device__ __forceinline__ void load_site(const LevReg<T>& R, const PassArgs<T>&
     }
   }
   window_of<T, D2>(R, i, j, x.c);
-  row_table(R.tab, k, x.row);
+  row_table(sm<T>() + R.tab, k, x.row);
 }
 
 // The heat-bath update of a loaded site.  The planes beyond a wall are the
-// slab's zeroed halo planes and carry zero band weights.
+// slab's zeroed halo planes and carry zero band weights.  FP32: the whole
+// window is loaded before the first sum, so that its loads share one latency.
 template <typename T, bool NOISE, bool D2>
 __device__ __forceinline__ T site_value(const LevReg<T>& R, const Site<T>& x) {
-  const T* vp = R.v + x.kz * R.pp;
+  const int vp = R.v + x.kz * R.pp;
   T acc = (T)0;
+  if constexpr (sizeof(T) == 4) {
+    T f[5][9];
 #pragma unroll
-  for (int dz = -2; dz <= 2; ++dz) {
-    T p1, p2;
-    if (dz == 0)
-      plane_sums<T, D2, false>(R, vp, x.c, &p1, &p2);
-    else
-      plane_sums<T, D2, true>(R, vp + dz * R.pp, x.c, &p1, &p2);
-    acc += x.row[dz + 2] * p1 + x.row[5 + dz + 2] * p2;
+    for (int d = 0; d < 5; ++d)
+#pragma unroll
+      for (int q = D2 ? 3 : 0; q < (D2 ? 6 : 9); ++q) {
+        if (d == 2 && q == 4) continue;
+        f[d][q] = sm<T>()[vp + (d - 2) * R.pp + x.c[q]];
+      }
+    asm volatile("" ::: "memory");
+#pragma unroll
+    for (int d = 0; d < 5; ++d) {
+      const T* w = f[d];
+      T p1, p2;
+      if (D2) {
+        p1 = R.a3 * w[3] + R.a3 * w[5];
+        p2 = R.b3 * w[3] + R.b3 * w[5];
+      } else {
+        p1 = R.a0 * w[0] + R.a1 * w[1] + R.a0 * w[2] + R.a3 * w[3] + R.a3 * w[5] + R.a0 * w[6] +
+             R.a1 * w[7] + R.a0 * w[8];
+        p2 = R.b0 * w[0] + R.b1 * w[1] + R.b0 * w[2] + R.b3 * w[3] + R.b3 * w[5] + R.b0 * w[6] +
+             R.b1 * w[7] + R.b0 * w[8];
+      }
+      if (d != 2) {
+        p1 += R.a4 * w[4];
+        p2 += R.b4 * w[4];
+      }
+      acc += x.row[d] * p1 + x.row[5 + d] * p2;
+    }
+  } else {
+#pragma unroll
+    for (int dz = -2; dz <= 2; ++dz) {
+      T p1, p2;
+      if (dz == 0)
+        plane_sums<T, D2, false>(R, vp, x.c, &p1, &p2);
+      else
+        plane_sums<T, D2, true>(R, vp + dz * R.pp, x.c, &p1, &p2);
+      acc += x.row[dz + 2] * p1 + x.row[5 + dz + 2] * p2;
+    }
   }
   T nv = (x.b - acc) * x.row[10];
   if (NOISE) nv += x.n * x.row[11];
+  return nv;
+}
+
+// ---- five lanes per site --------------------------------------------------------
+// A pass of a small class is latency: one warp alone works through its sites'
+// 45 loads and 100 operations.  Five consecutive lanes (six sites per warp)
+// each take one plane of the window, exchange the five terms by shuffles and
+// add them in the single lane's order.
+constexpr int kSplit = 5, kSplitSites = 32 / kSplit;
+
+template <typename T>
+struct SplitSite {
+  bool on;
+  int kz, c[9];
+  T z1, z2, rd, rs, b, n;
+};
+
+template <typename T, bool NOISE, bool D2>
+__device__ __forceinline__ T split_value(const LevReg<T>& R, const SplitSite<T>& x, int d, int lane0) {
+  T t = (T)0;
+  if (x.on) {
+    const int vp = R.v + (x.kz + d - 2) * R.pp;
+    T p1, p2;
+    plane_sums<T, D2, false>(R, vp, x.c, &p1, &p2);
+    if (d != 2) {
+      const T b1 = sm<T>()[vp + x.c[4]];
+      p1 += R.a4 * b1;
+      p2 += R.b4 * b1;
+    }
+    t = x.z1 * p1 + x.z2 * p2;
+  }
+  __syncwarp();
+  T acc = __shfl_sync(0xffffffffu, t, lane0);
+#pragma unroll
+  for (int e = 1; e < kSplit; ++e) acc += __shfl_sync(0xffffffffu, t, lane0 + e);
+  T nv = (x.b - acc) * x.rd;
+  if (NOISE) nv += x.n * x.rs;
   return nv;
 }
 
@@ -304,71 +388,136 @@ struct Remote {
   T* v[4];   // rank - 2, - 1, + 1, + 2: their plane z0, expressed from this CTA's plane z0
 };
 
-// `count` sweeps of a level: every colour class in turn, one thread per site,
-// a barrier after each class.  In the cluster a site within two planes of
-// another slab is also stored into that slab's halo.  The next pass's site
-// is loaded between arrival and release of the barrier.
-template <typename T, bool NOISE, bool D2>
-__device__ void sweeps(const View<T>& w, const PassArgs<T>& A, int count, int rank, int csize, bool cluster) {
+// `count` sweeps of a level: every colour class in turn, a thread (SPLIT: five
+// lanes) per site, a barrier after each class.  In the cluster a site within
+// two planes of another slab is also stored into that slab's halo.  What does
+// not depend on v is loaded off the critical path: when a class fits half of
+// the threads, the two halves take alternate passes, and one loads its next
+// pass while the other updates; else each thread loads its next site between
+// arrival and release of the barrier.  most: sites of the CTA's largest class.
+template <typename T, bool NOISE, bool D2, bool SPLIT>
+__device__ void sweeps(const View<T>& w, const PassArgs<T>& A, int count, int rank, int csize, bool cluster, int most) {
   const LevReg<T> R(w);
   Remote<T> rem;
-  if (cluster) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int d = q < 2 ? q - 2 : q - 1, r2 = rank + d;
-      rem.v[q] = nullptr;
-      if (r2 >= 0 && r2 < csize && min(r2 * R.P, w.L->nz) < min((r2 + 1) * R.P, w.L->nz))
-        rem.v[q] = cg::this_cluster().map_shared_rank(R.v, r2) - (long long)d * R.P * R.pp;
-    }
+  for (int q = 0; q < 4; ++q) {
+    const int d = q < 2 ? q - 2 : q - 1, r2 = rank + d;
+    rem.v[q] = nullptr;
+    if (cluster && r2 >= 0 && r2 < csize && min(r2 * R.P, w.L->nz) < min((r2 + 1) * R.P, w.L->nz))
+      rem.v[q] = cg::this_cluster().map_shared_rank(sm<T>() + R.v, r2) - (long long)d * R.P * R.pp;
   }
-  const int npass = count * R.ncol;
-  auto update = [&](const Site<T>& x) {
-    const T nv = site_value<T, NOISE, D2>(R, x);
-    const int pos = x.kz * R.pp + x.c[4];
-    R.v[pos] = nv;
-    if (cluster) {
-      // slab rank + d holds this plane when it is within two planes of it
+  // whether slab rank + d (q = 0..3: d = -2, -1, 1, 2) holds plane kz in its halo
+  auto near = [&](int q, int kz) { return q < 2 ? kz < 2 + (q - 1) * R.P : kz >= (q - 1) * R.P - 2; };
+  const int lane = threadIdx.x & 31;
+  const int part = SPLIT ? lane % kSplit : 0, lane0 = lane - part;   // SPLIT: this lane's plane
+  const bool idle = SPLIT && lane0 + kSplit > 32;                    // (lanes 30 and 31)
+  T* push = nullptr;   // SPLIT: lanes 1..4 of a site store into one neighbouring slab each
+  if (SPLIT && !idle) push = part == 1 ? rem.v[0] : part == 2 ? rem.v[1] : part == 3 ? rem.v[2] : part == 4 ? rem.v[3] : nullptr;
+  using Unit = std::conditional_t<SPLIT, SplitSite<T>, Site<T>>;
+  auto load = [&](const EngColour& cc, int q, int sweep, int u, Unit& x) {
+    if constexpr (SPLIT) {
+      Site<T> y;
+      load_site<T, NOISE, D2>(R, A, cc, q, sweep, u, y);
+      x.on = y.on;
+      if (!y.on) return;
+      x.kz = y.kz;
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int d = q < 2 ? q - 2 : q - 1;
-        const bool near = d < 0 ? x.kz < 2 + (d + 1) * R.P : x.kz >= d * R.P - 2;
-        if (rem.v[q] && near) rem.v[q][pos] = nv;
-      }
+      for (int e = 0; e < 9; ++e) x.c[e] = y.c[e];
+      const T* tr = sm<T>() + R.tab + 12 * (y.kz + R.z0);
+      x.z1 = tr[part];
+      x.z2 = tr[5 + part];
+      x.rd = tr[10];
+      x.rs = tr[11];
+      x.b = y.b;
+      x.n = y.n;
+    } else {
+      load_site<T, NOISE, D2>(R, A, cc, q, sweep, u, x);
     }
   };
-  int q = 0, sweep = A.first;
-  EngColour cc = R.col[0];
-  Site<T> x;
-  load_site<T, NOISE, D2>(R, A, cc, 0, sweep, threadIdx.x, x);
+  auto update = [&](const Unit& x) {
+    if constexpr (SPLIT) {   // every lane of the warp comes here
+      const T nv = split_value<T, NOISE, D2>(R, x, part, idle ? 0 : lane0);
+      if (!x.on) return;
+      const int pos = x.kz * R.pp + x.c[4];
+      if (part == 0)
+        sm<T>()[R.v + pos] = nv;
+      else if (push && near(part - 1, x.kz))
+        push[pos] = nv;
+    } else {
+      if (!x.on) return;
+      const T nv = site_value<T, NOISE, D2>(R, x);
+      const int pos = x.kz * R.pp + x.c[4];
+      sm<T>()[R.v + pos] = nv;
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (rem.v[q] && near(q, x.kz)) rem.v[q][pos] = nv;
+    }
+  };
+  // sites that one round of `threads` threads takes
+  auto sites_of = [](int threads) { return SPLIT ? (threads >> 5) * kSplitSites : threads; };
+  const int half_t = blockDim.x >> 1;
+  const bool halves = most <= sites_of(half_t);
+  const int tid = halves ? (int)threadIdx.x % half_t : (int)threadIdx.x;
+  const int group = halves ? (int)threadIdx.x / half_t : 0;
+  const int stride = sites_of(blockDim.x);
+  const int me = SPLIT ? (idle ? 1 << 24 : (tid >> 5) * kSplitSites + lane / kSplit) : tid;
+  const int npass = count * R.ncol;
+  int q = 0, sweep = A.first;   // class and sweep of pass p
+  auto colour = [&](int q) { return *reinterpret_cast<const EngColour*>(sm<unsigned char>() + R.col + q * (int)sizeof(EngColour)); };
+  EngColour cc = colour(0);
+  Unit x;
+  x.on = false;
+  if (group == 0 && npass > 0) load(cc, 0, sweep, me, x);
   for (int p = 0; p < npass; ++p) {
-    if (x.on) update(x);
-    for (int s = threadIdx.x + blockDim.x; s < cc.nsite; s += blockDim.x) {
-      load_site<T, NOISE, D2>(R, A, cc, q, sweep, s, x);
+    const int q1 = q + 1 == R.ncol ? 0 : q + 1, sweep1 = q1 == 0 ? sweep + 1 : sweep;
+    if (halves) {
+      if ((p & 1) == group) {
+        update(x);
+      } else if (p + 1 < npass) {
+        cc = colour(q1);
+        load(cc, q1, sweep1, me, x);
+      }
+      if (cluster) {
+        cg::this_cluster().barrier_arrive();
+        cg::this_cluster().barrier_wait();
+      } else {
+        __syncthreads();
+      }
+    } else {
       update(x);
+      if constexpr (!SPLIT) {   // (a SPLIT class fits one round)
+        for (int u = me + stride; u < cc.nsite; u += stride) {
+          load(cc, q, sweep, u, x);
+          update(x);
+        }
+      }
+      if (cluster) cg::this_cluster().barrier_arrive();
+      if (p + 1 < npass) {
+        cc = colour(q1);
+        load(cc, q1, sweep1, me, x);
+      }
+      if (cluster)
+        cg::this_cluster().barrier_wait();
+      else
+        __syncthreads();
     }
-    if (cluster) cg::this_cluster().barrier_arrive();
-    if (++q == R.ncol) {
-      q = 0;
-      ++sweep;
-    }
-    if (p + 1 < npass) {
-      cc = R.col[q];
-      load_site<T, NOISE, D2>(R, A, cc, q, sweep, threadIdx.x, x);
-    }
-    if (cluster)
-      cg::this_cluster().barrier_wait();
-    else
-      __syncthreads();
+    q = q1;
+    sweep = sweep1;
   }
 }
 
-template <typename T, bool NOISE>
+template <typename T, bool NOISE, bool D2>
 __device__ __forceinline__ void sweeps_any(const View<T>& w, const PassArgs<T>& A, int count, int rank, int csize,
                                            bool cluster) {
-  if (w.L->ny == 1)
-    sweeps<T, NOISE, true>(w, A, count, rank, csize, cluster);
-  else
-    sweeps<T, NOISE, false>(w, A, count, rank, csize, cluster);
+  int most = 0;
+  for (int q = 0; q < w.L->ncol; ++q) most = max(most, w.col[q].nsite);
+  if constexpr (sizeof(T) == 8) {   // (FP32: a site's row is short work for one lane)
+    if (most <= (int)(blockDim.x >> 5) * kSplitSites) {
+      sweeps<T, NOISE, D2, true>(w, A, count, rank, csize, cluster, most);
+      return;
+    }
+  }
+  sweeps<T, NOISE, D2, false>(w, A, count, rank, csize, cluster, most);
 }
 
 template <typename T>
@@ -382,7 +531,7 @@ __device__ void zero_local(const View<T>& w) {
 // planes: the x-y sums of a plane are formed once and kept for the five rows
 // that read them (9 shared loads per site instead of 45).
 template <typename T, bool D2>
-__device__ void residual_cols(const View<T>& w, const T* b, bool b_local, int boff, T* t) {
+__device__ void residual(const View<T>& w, const T* b, bool b_local, int boff, T* t) {
   const LevReg<T> R(w);
   const int cols = w.plane, np = w.z1 - w.z0;
   if (np <= 0) return;
@@ -403,7 +552,7 @@ __device__ void residual_cols(const View<T>& w, const T* b, bool b_local, int bo
       const int gidx = ((k + R.z0) * R.ny + j) * R.nx + i;
       const T bb = b_local ? b[gidx - boff] : ld_cg(b + gidx);
       T row[12];
-      row_table(R.tab, k + R.z0, row);
+      row_table(sm<T>() + R.tab, k + R.z0, row);
       T acc = (T)0;
 #pragma unroll
       for (int d = 0; d < 5; ++d) acc += row[d] * P1[d] + row[5 + d] * P2[d];
@@ -417,18 +566,10 @@ __device__ void residual_cols(const View<T>& w, const T* b, bool b_local, int bo
   }
 }
 
-template <typename T>
-__device__ __forceinline__ void residual(const View<T>& w, const T* b, bool b_local, int boff, T* t) {
-  if (w.L->ny == 1)
-    residual_cols<T, true>(w, b, b_local, boff, t);
-  else
-    residual_cols<T, false>(w, b, b_local, boff, t);
-}
-
 // b_c = P^T t on the coarse planes [Z0, Z1) of level Lc (tables on the fine
 // level Lf).  All taps of a site are loaded before they are summed.
 template <typename T, bool D2>
-__device__ void restrict_taps(const EngLevel<T>& Lf, const EngLevel<T>& Lc, const T* t, bool t_local, T* bc, int Z0,
+__device__ void restrict_to(const EngLevel<T>& Lf, const EngLevel<T>& Lc, const T* t, bool t_local, T* bc, int Z0,
                               int Z1) {
   constexpr int NY = D2 ? 1 : 3;
   const int nx = Lf.nx, ny = Lf.ny, ncx = Lc.nx, ncy = Lc.ny;
@@ -472,20 +613,11 @@ __device__ void restrict_taps(const EngLevel<T>& Lf, const EngLevel<T>& Lc, cons
   }
 }
 
-template <typename T>
-__device__ __forceinline__ void restrict_to(const EngLevel<T>& Lf, const EngLevel<T>& Lc, const T* t, bool t_local,
-                                            T* bc, int Z0, int Z1) {
-  if (Lf.ny == 1)
-    restrict_taps<T, true>(Lf, Lc, t, t_local, bc, Z0, Z1);
-  else
-    restrict_taps<T, false>(Lf, Lc, t, t_local, bc, Z0, Z1);
-}
-
 // v_f += P v_c on the local planes [z0-2, z1+2) of the fine view (halo
 // included).  A thread takes the pair of fine sites 2 I, 2 I + 1 of a row: the
 // even one is the coarse node I in x, the odd one the mean of I and I + 1.
 template <typename T, bool D2>
-__device__ void prolong_pairs(const View<T>& w, const EngLevel<T>& Lc, const T* vc, bool vc_local, int vc_z0) {
+__device__ void prolong_into(const View<T>& w, const EngLevel<T>& Lc, const T* vc, bool vc_local) {
   const EngLevel<T>& L = *w.L;
   const int nx = L.nx, ny = L.ny, rp = L.rp, pp = L.pp, half = L.half, z0 = w.z0;
   const int ncx = Lc.nx, ncy = Lc.ny, crp = Lc.rp, cpp = Lc.pp, chalf = Lc.half;
@@ -514,7 +646,7 @@ __device__ void prolong_pairs(const View<T>& w, const EngLevel<T>& Lc, const T* 
 #pragma unroll
       for (int a = 0; a < (D2 ? 1 : 2); ++a) {
         if (a == 1 && !yo) continue;
-        const int row = vc_local ? (kc - vc_z0 + 2) * cpp + yi[a] * crp : (kc * ncy + yi[a]) * ncx;
+        const int row = vc_local ? (kc + 2) * cpp + yi[a] * crp : (kc * ncy + yi[a]) * ncx;
         const T u0 = vc_local ? vc[row + xa] : ld_cg(vc + row + xa);
         const T u1 = vc_local ? vc[row + xb] : ld_cg(vc + row + xb);
         acc0 += wz * yw * (T)1 * u0;
@@ -526,15 +658,6 @@ __device__ void prolong_pairs(const View<T>& w, const EngLevel<T>& Lc, const T* 
     out[0] += acc0;
     out[half] += acc1;
   }
-}
-
-template <typename T>
-__device__ __forceinline__ void prolong_into(const View<T>& w, const EngLevel<T>& Lc, const T* vc, bool vc_local,
-                                             int vc_z0) {
-  if (w.L->ny == 1)
-    prolong_pairs<T, true>(w, Lc, vc, vc_local, vc_z0);
-  else
-    prolong_pairs<T, false>(w, Lc, vc, vc_local, vc_z0);
 }
 
 template <typename T>
@@ -563,38 +686,53 @@ __device__ void load_all(const View<T>& w, const T* g, T* dst) {
   for (int q = threadIdx.x; q < n; q += blockDim.x) dst[q] = ld_cg(g + q);
 }
 
-// Exact coarsest step in CTA 0: v = L^-T (L^-1 b + noise n), FP64.  Each
-// row of L^-1 b and each column of L^-T y is a dot product split over eight
-// consecutive lanes and reduced with shuffles.
+// Exact coarsest step: v = L^-T (L^-1 b + noise n), FP64.  Each row of L^-1 b
+// and each column of L^-T y is a dot product split over eight consecutive
+// lanes and reduced with shuffles.  With `spread` the rows (columns) are dealt
+// round-robin to the CTAs of the cluster, which take b from CTA 0, exchange y
+// and give v to CTA 0 through distributed shared memory (three cluster
+// barriers; the last one leaves v complete); else CTA 0 computes them all.
+// 216 unknowns (6^3): 27.3 us in CTA 0, 62 us noisy with its normals drawn by
+// one lane in eight.  On entry y[r] holds the normals of this CTA's rows.
 template <typename T, bool NOISE>
-__device__ void coarsest_step(const View<T>& w, int level, const T* b, double* y, Key key, unsigned long long cyc) {
+__device__ void coarsest_step(const View<T>& w, T* b, double* y, bool spread, int rank, int csize) {
   const EngLevel<T>& L = *w.L;
+  cg::cluster_group cl = cg::this_cluster();
   const int N = L.nx * L.ny * L.nz;
+  const int first = spread ? rank : 0, step = spread ? csize : 1;
   constexpr int G = 8;
-  const int span = (N * G + 31) / 32 * 32;   // whole warps: every lane reaches the shuffles
+  const int rows = (N - first + step - 1) / step;
+  const int span = (max(rows, 0) * G + 31) / 32 * 32;   // whole warps: every lane reaches the shuffles
+  if (spread) {
+    cl.sync();   // CTA 0's b is complete
+    if (rank != 0) {
+      const T* b0 = cl.map_shared_rank(b, 0);
+      for (int q = threadIdx.x; q < N; q += blockDim.x) b[q] = b0[q];
+      __syncthreads();
+    }
+  }
   for (int t = threadIdx.x; t < span; t += blockDim.x) {
-    const int r = t / G, g = t % G;
+    const int r = first + t / G * step, g = t % G;
     double acc = 0.0;
     if (r < N)
       for (int q = g; q <= r; q += G) acc += __ldg(L.Linv + (long long)r * N + q) * (double)b[q];
     acc += __shfl_xor_sync(0xffffffffu, acc, 4);
     acc += __shfl_xor_sync(0xffffffffu, acc, 2);
     acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-    if (r < N && g == 0) {
-      if (NOISE) {
-        const uint32_t c1 = (uint32_t)level | ((uint32_t)L.comp_id << 4) | (1u << 20);
-        double nn;
-        normal_of(eng_philox10(make_uint4((uint32_t)(r >> 2), c1, (uint32_t)cyc, (uint32_t)(cyc >> 32)), key.k0,
-                               key.k1),
-                  r & 3, &nn);
-        acc += nn;
-      }
-      y[r] = acc;
+    if (NOISE) {   // the row's lanes take their normal before one of them replaces it
+      const double nn = r < N && g == 0 ? y[r] : 0.0;
+      acc += __shfl_sync(0xffffffffu, nn, (threadIdx.x & 31) & ~(G - 1));
     }
+    if (r < N)
+      for (int c = g; c < step; c += G) (spread ? cl.map_shared_rank(y, c) : y)[r] = acc;
   }
-  __syncthreads();
+  if (spread)
+    cl.sync();
+  else
+    __syncthreads();
+  T* v = spread ? cl.map_shared_rank(w.v, 0) : w.v;
   for (int t = threadIdx.x; t < span; t += blockDim.x) {
-    const int col = t / G, g = t % G;
+    const int col = first + t / G * step, g = t % G;
     double acc = 0.0;
     if (col < N)
       for (int r = col + g; r < N; r += G) acc += __ldg(L.Linv + (long long)r * N + col) * y[r];
@@ -603,9 +741,13 @@ __device__ void coarsest_step(const View<T>& w, int level, const T* b, double* y
     acc += __shfl_xor_sync(0xffffffffu, acc, 1);
     if (col < N && g == 0) {
       const int i = col % L.nx, rr = col / L.nx;
-      w.v[w.loc(i, rr % L.ny, rr / L.ny)] = (T)acc;
+      v[w.loc(i, rr % L.ny, rr / L.ny)] = (T)acc;
     }
   }
+  if (spread)
+    cl.sync();
+  else
+    __syncthreads();
 }
 
 // Fills the colour-class table of the staged level L as seen by the CTA
@@ -646,6 +788,20 @@ template <typename T>
 __device__ void stage_noise(const EngParams<T>* P, const EngRun& run, unsigned char* smem, const EngLevel<T>* lev0,
                             const EngColour* col0, int rank, int csize, unsigned long long cyc) {
   const int lt = P->l0, lc = P->L - 1, ns = run.mu1 + run.mu2;
+  if (run.coarse_mode == SELM_COARSE_CHOLESKY) {   // the coarsest step's rows of this CTA
+    const EngLevel<T>& L = lev0[lc - lt];
+    const bool spread = lev0[0].cluster != 0;
+    const int N = L.nx * L.ny * L.nz, first = spread ? rank : 0, step = spread ? csize : 1;
+    double* y = reinterpret_cast<double*>(smem + P->y_off);
+    // from the last thread down: the level normals below start with the first
+    for (int t = blockDim.x - 1 - threadIdx.x; first + t * step < N && (spread || rank == 0); t += blockDim.x) {
+      const int r = first + t * step;
+      normal_of(eng_philox10(make_uint4((uint32_t)(r >> 2), (uint32_t)lc | ((uint32_t)L.comp_id << 4) | (1u << 20),
+                                        (uint32_t)cyc, (uint32_t)(cyc >> 32)),
+                             run.key.k0, run.key.k1),
+                r & 3, y + r);
+    }
+  }
   for (int l = lt; l <= lc; ++l) {
     if (P->nz_off[l] < 0 || (l == lc && run.coarse_mode == SELM_COARSE_CHOLESKY)) continue;
     const EngLevel<T>& L = lev0[l - lt];
@@ -682,7 +838,7 @@ __device__ void stage_noise(const EngParams<T>* P, const EngRun& run, unsigned c
   }
 }
 
-template <typename T, bool NOISE>
+template <typename T, bool NOISE, bool D2>
 __global__ void __launch_bounds__(EngThreads<T>::value, 1) k_coarse_engine(const EngParams<T>* __restrict__ P, EngRun run) {
   extern __shared__ __align__(16) unsigned char smem[];
   cg::cluster_group cl = cg::this_cluster();
@@ -812,10 +968,10 @@ __global__ void __launch_bounds__(EngThreads<T>::value, 1) k_coarse_engine(const
     PassArgs<T> A;
     A.level = l;
     A.first = first;
-    A.b = b;
+    A.gb = L.gb;
     A.b_local = blocal;
-    A.boff = boff;
-    A.noise = NOISE && P->nz_off[l] >= 0 ? reinterpret_cast<const T*>(smem + P->nz_off[l]) : nullptr;
+    A.sb = blocal ? sm_at(b) - boff : 0;
+    A.noise = NOISE && P->nz_off[l] >= 0 ? P->nz_off[l] / (int)sizeof(T) : -1;
     A.nstride = L.P * L.nx * L.ny;
     A.c1 = (uint32_t)l | ((uint32_t)L.comp_id << 4);
     A.key = key;
@@ -823,6 +979,7 @@ __global__ void __launch_bounds__(EngThreads<T>::value, 1) k_coarse_engine(const
     return A;
   };
 
+  for (int l = lt; l <= lc; ++l) zero_local(make_view(sl_at(l), smem, rank, sl_at(l).cluster != 0));
   pdl_wait();   // everything above reads only the plan and the counter
   // ---- down leg over the cluster levels ----
   int l = lt;
@@ -830,15 +987,14 @@ __global__ void __launch_bounds__(EngThreads<T>::value, 1) k_coarse_engine(const
     const EngLevel<T>& L = sl_at(l);
     const EngLevel<T>& Lc = sl_at(l + 1);
     View<T> w = view_of(l, true);
-    zero_local(w);
     // b of the owned planes in shared memory when the plan has room for it
     const bool bl = L.sb >= 0;
     const T* bsrc = bl ? (const T*)(smem + L.sb) : L.gb;
     const int boff = bl ? w.z0 * w.plane : 0;
     if (bl) load_owned(w, L.gb, (T*)(smem + L.sb));
     cl.sync();
-    sweeps_any<T, NOISE>(w, pass_args(l, 0, bsrc, bl, boff), mu1, rank, csize, true);
-    residual(w, bsrc, bl, boff, L.gt);
+    sweeps_any<T, NOISE, D2>(w, pass_args(l, 0, bsrc, bl, boff), mu1, rank, csize, true);
+    residual<T, D2>(w, bsrc, bl, boff, L.gt);
     cl.sync();
     // the coarse planes of the restriction are split over the cluster's CTAs
     // (also when the coarse level is held by CTA 0: it reads them back)
@@ -847,7 +1003,7 @@ __global__ void __launch_bounds__(EngThreads<T>::value, 1) k_coarse_engine(const
     const int Z1 = min(Z0 + Pc, Lc.nz);
     // into the first level held by CTA 0: its shared b, through distributed shared memory
     T* bdst = Lc.cluster ? Lc.gb : cl.map_shared_rank(reinterpret_cast<T*>(smem + Lc.sb), 0);
-    restrict_to(L, Lc, L.gt, false, bdst, Z0, Z1);
+    restrict_to<T, D2>(L, Lc, L.gt, false, bdst, Z0, Z1);
     cl.sync();
   }
   const int lsingle = l;   // first level held by CTA 0 alone
@@ -856,6 +1012,11 @@ __global__ void __launch_bounds__(EngThreads<T>::value, 1) k_coarse_engine(const
     cl.sync();
     if (rank != 0) return;
   }
+  // the coarsest step is spread over the cluster: the other CTAs wait in it
+  const bool spread = lsingle > lt && run.coarse_mode == SELM_COARSE_CHOLESKY;
+  if (spread && rank != 0)
+    coarsest_step<T, NOISE>(view_of(lc, false), (T*)(smem + sl_at(lc).sb), (double*)(smem + P->y_off), true, rank,
+                            csize);
   if (rank == 0) {
     // ---- single-CTA part: levels lsingle .. lc and back ----
     if (lsingle == lt) {   // b from global only when no cluster level restricted into it
@@ -866,31 +1027,29 @@ __global__ void __launch_bounds__(EngThreads<T>::value, 1) k_coarse_engine(const
       const EngLevel<T>& L = sl_at(k);
       View<T> w = view_of(k, false);
       T* b = (T*)(smem + L.sb);
-      zero_local(w);
       __syncthreads();
       if (k == lc && run.coarse_mode == SELM_COARSE_CHOLESKY) {
-        coarsest_step<T, NOISE>(w, k, b, (double*)(smem + P->y_off), key, cyc);
-        __syncthreads();
+        coarsest_step<T, NOISE>(w, b, (double*)(smem + P->y_off), spread, rank, csize);
         break;
       }
-      sweeps_any<T, NOISE>(w, pass_args(k, 0, b, true, 0), mu1, 0, 1, false);
+      sweeps_any<T, NOISE, D2>(w, pass_args(k, 0, b, true, 0), mu1, 0, 1, false);
       if (k == lc) {
-        sweeps_any<T, NOISE>(w, pass_args(k, mu1, b, true, 0), mu2, 0, 1, false);
+        sweeps_any<T, NOISE, D2>(w, pass_args(k, mu1, b, true, 0), mu2, 0, 1, false);
         break;
       }
       const EngLevel<T>& Lc = sl_at(k + 1);
-      residual(w, b, true, 0, (T*)(smem + L.st));
+      residual<T, D2>(w, b, true, 0, (T*)(smem + L.st));
       __syncthreads();
-      restrict_to(L, Lc, (const T*)(smem + L.st), true, (T*)(smem + Lc.sb), 0, Lc.nz);
+      restrict_to<T, D2>(L, Lc, (const T*)(smem + L.st), true, (T*)(smem + Lc.sb), 0, Lc.nz);
       __syncthreads();
     }
     for (int k = lc - 1; k >= lsingle; --k) {
       const EngLevel<T>& L = sl_at(k);
       const EngLevel<T>& Lc = sl_at(k + 1);
       View<T> w = view_of(k, false);
-      prolong_into(w, Lc, (const T*)(smem + Lc.sv), true, 0);
+      prolong_into<T, D2>(w, Lc, (const T*)(smem + Lc.sv), true);
       __syncthreads();
-      sweeps_any<T, NOISE>(w, pass_args(k, mu1, (const T*)(smem + L.sb), true, 0), mu2, 0, 1, false);
+      sweeps_any<T, NOISE, D2>(w, pass_args(k, mu1, (const T*)(smem + L.sb), true, 0), mu2, 0, 1, false);
     }
     {   // the engine's result, or the hand-off to the cluster's prolongation
       View<T> w = view_of(lsingle, false);
@@ -905,7 +1064,7 @@ __global__ void __launch_bounds__(EngThreads<T>::value, 1) k_coarse_engine(const
     const EngLevel<T>& Lc = sl_at(k + 1);
     View<T> w = view_of(k, true);
     if (Lc.cluster) {
-      prolong_into(w, Lc, Lc.gv, false, 0);
+      prolong_into<T, D2>(w, Lc, Lc.gv, false);
     } else {
       // the coarse level is held by CTA 0, which still has its v in shared
       // memory; the other CTAs first copy the coarse planes that their slab and
@@ -931,11 +1090,11 @@ __global__ void __launch_bounds__(EngThreads<T>::value, 1) k_coarse_engine(const
         }
         __syncthreads();
       }
-      prolong_into(w, Lc, (const T*)wc.v, true, 0);
+      prolong_into<T, D2>(w, Lc, (const T*)wc.v, true);
     }
     cl.sync();
     const bool bl = L.sb >= 0;   // staged on the way down, untouched since
-    sweeps_any<T, NOISE>(w, pass_args(k, mu1, bl ? (const T*)(smem + L.sb) : L.gb, bl, bl ? w.z0 * w.plane : 0), mu2,
+    sweeps_any<T, NOISE, D2>(w, pass_args(k, mu1, bl ? (const T*)(smem + L.sb) : L.gb, bl, bl ? w.z0 * w.plane : 0), mu2,
                          rank, csize, true);
     store_owned(w, L.gv);
     cl.sync();
@@ -997,7 +1156,9 @@ bool try_plan(const LevelDev* levs, int L, int l0, int C, bool stage_b, int swee
       EngLevel<T>& e = p.comp[c].lev[l];
       const long long sites = (long long)d.nx * d.ny * d.nz;
       if (sites >= (1ll << 24)) return false;   // rank decode uses float reciprocals
-      const bool single = single_started || l == L - 1 || sites <= kEngSingleMaxSites || C == 1;
+      for (const double* wt : {d.w1, d.w2})   // the passes keep one weight per kind of neighbour
+        if (wt[0] != wt[2] || wt[0] != wt[6] || wt[0] != wt[8] || wt[1] != wt[7] || wt[3] != wt[5]) return false;
+      const bool single = single_started || l == L - 1 || sites <= eng_single_sites<T>() || C == 1;
       if (single) single_started = true;
       e.cluster = single ? 0 : 1;
       if (e.cluster) any_cluster = true;
@@ -1152,7 +1313,8 @@ bool raise_smem_limit() {
     cudaGetLastError();
     return false;
   }
-  for (auto fn : {k_coarse_engine<T, true>, k_coarse_engine<T, false>}) {
+  for (auto fn : {k_coarse_engine<T, true, false>, k_coarse_engine<T, false, false>, k_coarse_engine<T, true, true>,
+                  k_coarse_engine<T, false, true>}) {
     cudaFuncAttributes fa{};
     if (cudaFuncGetAttributes(&fa, fn) != cudaSuccess ||
         cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes) !=
@@ -1208,7 +1370,8 @@ bool plan_coarse_engine(const LevelDev* levs, int L, void* const* gb, void* cons
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int nclusters = 0;
-        if (cudaOccupancyMaxActiveClusters(&nclusters, k_coarse_engine<T, true>, &cfg) == cudaSuccess && nclusters >= 1)
+        if (cudaOccupancyMaxActiveClusters(
+                &nclusters, levs[0].c[0].ny == 1 ? k_coarse_engine<T, true, true> : k_coarse_engine<T, true, false>, &cfg) == cudaSuccess && nclusters >= 1)
           return true;
         cudaGetLastError();
         return false;
@@ -1262,8 +1425,11 @@ cudaError_t launch_coarse_engine(const EnginePlanT<T>& plan, int mu1, int mu2, i
   cfg.attrs = attr;
   cfg.numAttrs = 2;
   prof::Scope ps(SELM_K_COARSE_SWEEP, st);
-  if (noise) return cudaLaunchKernelEx(&cfg, k_coarse_engine<T, true>, plan.dev, run);
-  return cudaLaunchKernelEx(&cfg, k_coarse_engine<T, false>, plan.dev, run);
+  const bool d2 = plan.params.comp[0].lev[plan.params.l0].ny == 1;
+  if (noise && d2) return cudaLaunchKernelEx(&cfg, k_coarse_engine<T, true, true>, plan.dev, run);
+  if (noise) return cudaLaunchKernelEx(&cfg, k_coarse_engine<T, true, false>, plan.dev, run);
+  if (d2) return cudaLaunchKernelEx(&cfg, k_coarse_engine<T, false, true>, plan.dev, run);
+  return cudaLaunchKernelEx(&cfg, k_coarse_engine<T, false, false>, plan.dev, run);
 }
 
 template bool plan_coarse_engine<float>(const LevelDev*, int, void* const*, void* const*, void* const*, void*,

@@ -11,7 +11,14 @@
 namespace selm {
 
 // Levels with at most this many sites per component are held by one CTA.
-constexpr long long kEngSingleMaxSites = 8192;
+// FP32: a pass of a 16^3 level takes 0.7 us in one CTA and 1.1 us over the
+// cluster, whose barrier costs more than the work it divides.  FP64: two lanes
+// per clock and SM bound a pass (16^3: 10.9 us in one CTA, 4.2 us over 16; 32^2
+// in 2-D: 2.5 and 1.1 us), so all but the smallest levels are divided.
+template <typename T>
+constexpr long long eng_single_sites() {
+  return sizeof(T) == 4 ? 8192 : 256;
+}
 
 template <typename T>
 struct EngLevel {
