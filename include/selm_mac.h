@@ -111,8 +111,9 @@ selm_status selm_mac_divergence(selm_mac* h, const double* u, double* div, void*
 selm_status selm_mac_gradient(selm_mac* h, const double* p, double* grad, void* stream);
 /* out = P~ u (adjoint = 0) or P~^T u = W P~ W^-1 u (adjoint = 1); out may
    equal u.  The pressure L phi = D u (phi of zero volume mean) is solved by
-   conjugate gradients on diag(vol) L (Jacobi preconditioned, FP64) to
-   proj_tol; iters / resid (optional HOST pointers) receive the iteration
+   FP64 conjugate gradients on diag(vol) L to proj_tol, preconditioned by the
+   operator's spectral solve (3-D, n a power of two up to 64), else by its
+   diagonal; iters / resid (optional HOST pointers) receive the iteration
    count and relative residual (synchronises the stream). */
 selm_status selm_mac_project(selm_mac* h, const double* u, double* out, int adjoint, int* iters, double* resid,
                              void* stream);

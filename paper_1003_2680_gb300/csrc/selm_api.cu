@@ -503,23 +503,23 @@ selm_status fac_solve(selm_mg* h, Sys& s, double* z, const double* b, double tol
   }
 }
 
-// The projection's pressure problem by FP64 iterative refinement around the
-// spectral inner solve (Algorithm 1's iteration with the exact FP32 solve of
-// the uniform channel's Neumann operator in place of the V-cycle): residual
-// r = b - A phi in FP64, delta = A^-1 r in FP32 (FFT along x, y; Thomas along
-// z), phi += delta, until ||r|| <= tol ||b||.
-selm_status spectral_fac_solve(selm_mg* h, double* phi, const double* b, double tol, int max_cycles, int* cycles,
-                               double* rel_out, cudaStream_t st) {
-  Sys& s = h->pres;
+// FP64 iterative refinement around the spectral inner solve (Algorithm 1's
+// iteration with the exact FP32 solve of the uniform channel's operator in
+// place of the V-cycle): residual r = b - A z in FP64, delta = A^-1 r in FP32
+// (FFT along x, y; Thomas along z), z += delta, until ||r|| <= tol ||b||.  It
+// ends short of tol (SELM_ENOCONV) where the residual no longer halves below
+// `floor` ||b||, the rounding of its own evaluation (0: only max_cycles ends it).
+selm_status spectral_fac_solve(selm_mg* h, Sys& s, double* z, const double* b, double tol, int max_cycles, double floor,
+                               void* spectrum, int* cycles, double* rel_out, cudaStream_t st) {
   double* nb = h->red + 0;
   double* nr = h->red + 1;
   CK(cudaMemsetAsync(nb, 0, 2 * sizeof(double), st));
   CK(launch_norm2(s.lev[0].size, b, nb, st));
   *cycles = 0;
-  double bn = 0.0;
+  double bn = 0.0, rel_prev = -1.0;
   for (int cyc = 0;; ++cyc) {
     if (cyc > 0) CK(cudaMemsetAsync(nr, 0, sizeof(double), st));
-    selm_status r = outer_residual(h, s, phi, b, s.b[0], nr, st);
+    selm_status r = outer_residual(h, s, z, b, s.b[0], nr, st);
     if (r != SELM_OK) return r;
     CK(cudaEventRecord(h->ev_norm, st));
     double bn2 = 0.0, rn2 = 0.0;
@@ -527,7 +527,7 @@ selm_status spectral_fac_solve(selm_mg* h, double* phi, const double* b, double 
     if (r != SELM_OK) return r;
     if (cyc == 0) {
       if (bn2 == 0.0) {
-        CK(cudaMemsetAsync(phi, 0, (size_t)s.lev[0].size * sizeof(double), st));
+        CK(cudaMemsetAsync(z, 0, (size_t)s.lev[0].size * sizeof(double), st));
         if (rel_out) *rel_out = 0.0;
         return SELM_OK;
       }
@@ -539,13 +539,14 @@ selm_status spectral_fac_solve(selm_mg* h, double* phi, const double* b, double 
       *cycles = cyc;
       return SELM_OK;
     }
-    if (cyc >= max_cycles) {
+    if (cyc >= max_cycles || (rel_prev >= 0.0 && rel <= floor && rel > 0.5 * rel_prev)) {
       *cycles = cyc;
-      h->err = "spectral pressure solve did not converge";
+      h->err = "spectral solve did not converge";
       return SELM_ENOCONV;
     }
-    CK(spectral_pressure_solve(s.lev[0], (const float*)s.b[0], (float*)s.v[0], h->spec, st));
-    r = outer_update(h, s, phi, s.v[0], st);
+    rel_prev = rel;
+    CK(spectral_inner_solve(s.lev[0], (const float*)s.b[0], (float*)s.v[0], spectrum, st));
+    r = outer_update(h, s, z, s.v[0], st);
     if (r != SELM_OK) return r;
   }
 }
@@ -566,7 +567,8 @@ selm_status project(selm_mg* h, double* w, int* cycles, cudaStream_t st, int slo
   if (slot < 0) CK(cudaMemsetAsync(phi, 0, (size_t)np_ * sizeof(double), st));
   double rel = 0.0;
   selm_status r = h->spectral && h->spec
-                      ? spectral_fac_solve(h, phi, h->prhs, h->d.proj_tol, h->d.max_cycles, cycles, &rel, st)
+                      ? spectral_fac_solve(h, h->pres, phi, h->prhs, h->d.proj_tol, h->d.max_cycles, 0.0, h->spec,
+                                           cycles, &rel, st)
                       : fac_solve(h, h->pres, phi, h->prhs, h->d.proj_tol, h->d.max_cycles, cycles, &rel, st);
   if (r != SELM_OK) return r;
   CK(launch_grad_sub(h->vel.lev[0], w, phi, st));
@@ -621,6 +623,12 @@ int engine_first_level(const selm_mg* h, const Sys& s) {
 namespace selm {
 
 selm_status chain_advance(selm_mg* h, int ncycles, cudaStream_t st) { return chain_cycles(h, ncycles, st); }
+
+selm_status spectral_velocity_solve(selm_mg* h, double* z, const double* b, double tol, double floor, void* spectrum,
+                                    double* rel, cudaStream_t st) {
+  int cycles = 0;
+  return spectral_fac_solve(h, h->vel, z, b, tol, h->d.max_cycles, floor, spectrum, &cycles, rel, st);
+}
 
 size_t footprint_with_host(const selm_mg_desc& d, const HostSystem& host, size_t extra_bytes) {
   Sys vel;
@@ -836,7 +844,7 @@ selm_status selm_mg_create(const selm_mg_desc* desc, void* stream, selm_mg** out
   if (h->has_pres) {
     h->phi = (double*)(h->ws + p.phi_off);
     h->prhs = (double*)(h->ws + p.prhs_off);
-    if (p.spec_bytes > 0 && spectral_pressure_supported(h->pres.lev[0])) {
+    if (p.spec_bytes > 0 && spectral_supported(h->pres.lev[0])) {
       h->spec = h->ws + p.spec_off;
       h->spectral = true;
     }

@@ -153,6 +153,12 @@ size_t footprint_with_host(const selm_mg_desc& d, const HostSystem& host, size_t
 selm_status vcycle_level(selm_mg* h, Sys& s, int level, bool noise, const unsigned long long* cyc, cudaStream_t st);
 // `ncycles` stochastic FAC cycles of the handle's chain xi (b = 0).
 selm_status chain_advance(selm_mg* h, int ncycles, cudaStream_t st);
+// z from its value to ||b - A z|| <= tol ||b|| for the velocity system by the
+// spectral inner solve (spectral_supported(), FP32 inner precision);
+// `spectrum`: spectral_bytes() of scratch.  SELM_ENOCONV with *rel set when it
+// stagnates below `floor` or runs out of cycles.
+selm_status spectral_velocity_solve(selm_mg* h, double* z, const double* b, double tol, double floor, void* spectrum,
+                                    double* rel, cudaStream_t st);
 // Frees the Stokes scratch (selm_stokes.cu).
 void stokes_release(selm_mg* h);
 

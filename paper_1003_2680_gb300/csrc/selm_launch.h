@@ -108,13 +108,20 @@ cudaError_t launch_grad_sub(const LevelDev& Lv, double* w, const double* phi, cu
 
 cudaError_t launch_philox(const uint32_t* ctr, Key key, uint32_t* out, int n, cudaStream_t st);
 
-// Spectral inner solve of the uniform channel's Neumann pressure problem
-// (selm_spectral.cu): delta = A^-1 r up to FP32 rounding (FFT along x and y,
-// Thomas along z); `spectrum`: spectral_pressure_bytes() of scratch.
-bool spectral_pressure_supported(const LevelDev& L0);
-size_t spectral_pressure_bytes(const LevelDev& L0);
-cudaError_t spectral_pressure_solve(const LevelDev& L0, const float* r, float* delta, void* spectrum,
-                                    cudaStream_t st);
+// Spectral inner solves of the uniform channel (selm_spectral.cu): delta =
+// A^-1 r up to FP32 rounding (FFT along x and y, Thomas along z) for the
+// Neumann pressure problem or the no-slip velocity components; `spectrum`:
+// spectral_bytes() of scratch.
+bool spectral_supported(const LevelDev& L0);
+size_t spectral_bytes(const LevelDev& L0);
+cudaError_t spectral_inner_solve(const LevelDev& L0, const float* r, float* delta, void* spectrum, cudaStream_t st);
+// The same for the staggered composite grid's pressure operator
+// S = diag(vol) D G (n base cells per edge, K refined rows): z = S^-1 r up to
+// FP32 rounding, r and z in FP64; *rr (device) = ||r||^2.
+bool mac_spectral_supported(int dim, int n, int K);
+size_t mac_spectral_bytes(int n, int K);
+cudaError_t mac_spectral_solve(int n, int K, const double* r, double* z, const double* rr, void* spectrum,
+                               cudaStream_t st);
 
 // ---- batched FAC cycles as one persistent launch ----------------------------
 // One system of a batch as the persistent launch sees it (device pointers of

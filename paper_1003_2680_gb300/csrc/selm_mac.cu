@@ -164,6 +164,16 @@ __global__ void __launch_bounds__(kThreads) k_dot_part(long long n, const double
   if (threadIdx.x == 0) part[blockIdx.x] = a;
 }
 
+// Per-block partial sums of x.
+__global__ void __launch_bounds__(kThreads) k_sum_part(long long n, const double* __restrict__ x,
+                                                      double* __restrict__ part) {
+  double a = 0.0;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+    a += x[i];
+  a = block_sum(a);
+  if (threadIdx.x == 0) part[blockIdx.x] = a;
+}
+
 // Heat-bath update of one colour class (Eq. equ_R_GS with the noise term of
 // Eq. equ_def_Q_GS): v_i = (b_i - sum_{j != i} a_ij v_j) / a_ii
 //                          + sigma n_i / sqrt(a_ii).
@@ -532,6 +542,9 @@ __global__ void __launch_bounds__(kThreads) k_cg_mv(SellDev S, const double* __r
   if (threadIdx.x == 0) part[blockIdx.x] = acc;
 }
 
+// (JACOBI: z = r / diag(S) and its r.z with the update; else z follows from the
+// spectral columns.)
+template <bool JACOBI>
 __global__ void __launch_bounds__(kThreads) k_cg_update(long long n, int nb, const double* __restrict__ part_pq,
                                                        const double* __restrict__ sc, int old,
                                                        double* __restrict__ x, double* __restrict__ r,
@@ -546,15 +559,17 @@ __global__ void __launch_bounds__(kThreads) k_cg_update(long long n, int nb, con
     x[i] += alpha * p[i];
     const double ri = r[i] - alpha * q[i];
     r[i] = ri;
-    const double zi = ri * minv[i];
-    z[i] = zi;
-    rz += ri * zi;
+    if (JACOBI) {
+      const double zi = ri * minv[i];
+      z[i] = zi;
+      rz += ri * zi;
+    }
     rr += ri * ri;
   }
-  rz = block_sum(rz);
+  if (JACOBI) rz = block_sum(rz);
   rr = block_sum(rr);
   if (threadIdx.x == 0) {
-    part[blockIdx.x] = rz;
+    if (JACOBI) part[blockIdx.x] = rz;
     part[kRedBlocks + blockIdx.x] = rr;
   }
 }
@@ -757,6 +772,7 @@ struct selm_mac {
   double* part_rows = nullptr;       // one partial per block of the outer residual's rows
   double* sc = nullptr;              // device scalars
   double* host_sc = nullptr;         // pinned host copy
+  void* spec = nullptr;              // spectra of the pressure solve (null: Jacobi preconditioner)
   double *cg_x = nullptr, *cg_r = nullptr, *cg_z = nullptr, *cg_p = nullptr, *cg_q = nullptr;
   double *fw = nullptr, *fw2 = nullptr, *fine_buf = nullptr, *pv = nullptr;
   int max_np = 0;
@@ -1070,14 +1086,108 @@ selm_status solve(selm_mac* h, double* z, const double* b, double tol, int max_c
   return SELM_OK;
 }
 
+// x = 0, r = vol rhs less its mean: the sum of a consistent right-hand side is
+// rounding, which no iteration can reduce, and not small against one that is
+// itself rounding (the divergence of an already projected field).
+selm_status pressure_rhs(selm_mac* h, const double* rhs, cudaStream_t st) {
+  const long long n = h->n_cells;
+  const unsigned nb = red_blocks(n), eb = blocks_for(n);
+  k_scale<false><<<eb, kThreads, 0, st>>>(n, rhs, h->vol, h->cg_r);
+  MCK(cudaMemsetAsync(h->cg_x, 0, n * sizeof(double), st));
+  k_sum_part<<<nb, kThreads, 0, st>>>(n, h->cg_r, h->part);
+  k_reduce<<<1, kThreads, 0, st>>>(h->part, (int)nb, h->sc + 6);
+  k_sub_scalar<<<eb, kThreads, 0, st>>>(n, h->cg_r, h->sc + 6, 1.0 / (double)n);
+  MCK(cudaGetLastError());
+  return SELM_OK;
+}
+
+// phi -> its representative of zero volume mean.
+selm_status zero_mean(selm_mac* h, cudaStream_t st) {
+  const long long n = h->n_cells;
+  const unsigned nb = red_blocks(n);
+  prof::Scope ps(SELM_K_PROJECTION, st);
+  k_dot_part<<<nb, kThreads, 0, st>>>(n, h->cg_x, h->vol, h->part);
+  k_reduce<<<1, kThreads, 0, st>>>(h->part, (int)nb, h->sc + 6);
+  k_sub_scalar<<<blocks_for(n), kThreads, 0, st>>>(n, h->cg_x, h->sc + 6, 1.0 / h->total_vol);
+  MCK(cudaGetLastError());
+  return SELM_OK;
+}
+
+// The same conjugate gradients with the spectral solve of the composite
+// operator (FP32, selm_spectral.cu) as the preconditioner: exact up to FP32
+// rounding, so the FP64 recurrence gains about five digits per iteration
+// (64^3 + 8 rows to 1e-13: 3 iterations instead of 512, 0.59 ms instead of 18).
+// The residual and all inner products stay FP64.  *done = false when the
+// residual stops falling short of proj_tol.
+selm_status pressure_solve_spectral(selm_mac* h, const double* rhs, int* iters, double* resid, bool* done,
+                                    cudaStream_t st) {
+  const long long n = h->n_cells;
+  const unsigned nb = red_blocks(n), eb = blocks_for(n);
+  auto precondition = [&]() {   // z = S^-1 r, r.z partials
+    cudaError_t e = mac_spectral_solve(h->d.n, h->d.K, h->cg_r, h->cg_z, h->sc + 3, h->spec, st);
+    if (e != cudaSuccess) return e;
+    prof::Scope ps(SELM_K_PROJECTION, st);
+    k_dot_part<<<nb, kThreads, 0, st>>>(n, h->cg_r, h->cg_z, h->part2);
+    return cudaGetLastError();
+  };
+  {
+    prof::Scope ps(SELM_K_PROJECTION, st);
+    MRET(pressure_rhs(h, rhs, st));
+    k_dot_part<<<nb, kThreads, 0, st>>>(n, h->cg_r, h->cg_r, h->part);
+    k_reduce<<<1, kThreads, 0, st>>>(h->part, (int)nb, h->sc + 3);
+    MCK(cudaGetLastError());
+  }
+  MCK(cudaMemcpyAsync(h->host_sc, h->sc, 8 * sizeof(double), cudaMemcpyDeviceToHost, st));
+  MCK(cudaStreamSynchronize(st));
+  const double bn = std::sqrt(h->host_sc[3]);
+  const double tol = h->d.proj_tol;
+  double rn = bn;
+  int it = 0, idle = 0;
+  *done = false;
+  while (bn > 0.0 && rn > tol * bn) {
+    const int old = it & 1;   // r.z of this iteration in sc[old]
+    MCK(precondition());
+    {
+      prof::Scope ps(SELM_K_PROJECTION, st);
+      if (it == 0) {
+        k_reduce<<<1, kThreads, 0, st>>>(h->part2, (int)nb, h->sc + old);
+        MCK(cudaMemcpyAsync(h->cg_p, h->cg_z, n * sizeof(double), cudaMemcpyDeviceToDevice, st));
+      } else {
+        k_cg_dir<<<nb, kThreads, 0, st>>>(n, (int)nb, h->part2, h->sc, old ^ 1, h->cg_z, h->cg_p);
+      }
+      k_cg_mv<<<nb, kThreads, 0, st>>>(h->S, h->cg_p, h->cg_q, h->part);
+      k_cg_update<false><<<nb, kThreads, 0, st>>>(n, (int)nb, h->part, h->sc, old, h->cg_x, h->cg_r, h->cg_p, h->cg_q,
+                                                  nullptr, nullptr, h->part2);
+      k_reduce<<<1, kThreads, 0, st>>>(h->part2 + kRedBlocks, (int)nb, h->sc + 3);
+      MCK(cudaGetLastError());
+    }
+    ++it;
+    MCK(cudaMemcpyAsync(h->host_sc, h->sc, 8 * sizeof(double), cudaMemcpyDeviceToHost, st));
+    MCK(cudaStreamSynchronize(st));
+    const double rn_new = std::sqrt(h->host_sc[3]);
+    idle = rn_new < 0.5 * rn ? 0 : idle + 1;   // (an iteration gains several digits; NaN counts as idle)
+    rn = rn_new;
+    if (idle == 3) return SELM_OK;
+  }
+  *done = true;
+  MRET(zero_mean(h, st));
+  if (iters) *iters = it;
+  if (resid) *resid = bn > 0.0 ? rn / bn : 0.0;
+  return SELM_OK;
+}
+
 // phi with L phi = rhs (cells), zero volume mean, by PCG on diag(vol) L.
 selm_status pressure_solve(selm_mac* h, const double* rhs, int* iters, double* resid, cudaStream_t st) {
+  if (h->spec) {
+    bool done = false;
+    MRET(pressure_solve_spectral(h, rhs, iters, resid, &done, st));
+    if (done) return SELM_OK;
+  }
   const long long n = h->n_cells;
   const unsigned nb = red_blocks(n), eb = blocks_for(n);
   {
     prof::Scope ps(SELM_K_PROJECTION, st);
-    k_scale<false><<<eb, kThreads, 0, st>>>(n, rhs, h->vol, h->cg_r);      // r = vol rhs (x = 0)
-    MCK(cudaMemsetAsync(h->cg_x, 0, n * sizeof(double), st));
+    MRET(pressure_rhs(h, rhs, st));
     k_cg_start<<<nb, kThreads, 0, st>>>(n, h->cg_r, h->minv, h->cg_z, h->cg_p, h->part);
     k_cg_reduce2<<<1, kThreads, 0, st>>>(h->part, (int)nb, h->sc);
     k_cg_shift<<<1, 1, 0, st>>>(h->sc);
@@ -1101,7 +1211,7 @@ selm_status pressure_solve(selm_mac* h, const double* rhs, int* iters, double* r
       const int old = k & 1;
       cudaError_t e = launch_pdl(k_cg_mv, nb, kThreads, s2, h->S, (const double*)h->cg_p, h->cg_q, h->part);
       if (e == cudaSuccess)
-        e = launch_pdl(k_cg_update, nb, kThreads, s2, n, (int)nb, (const double*)h->part, (const double*)h->sc, old,
+        e = launch_pdl(k_cg_update<true>, nb, kThreads, s2, n, (int)nb, (const double*)h->part, (const double*)h->sc, old,
                        h->cg_x, h->cg_r, (const double*)h->cg_p, (const double*)h->cg_q, h->minv, h->cg_z,
                        h->part2);
       if (e == cudaSuccess)
@@ -1140,13 +1250,7 @@ selm_status pressure_solve(selm_mac* h, const double* rhs, int* iters, double* r
     MCK(cudaStreamSynchronize(st));
     rn = std::sqrt(h->host_sc[3]);
   }
-  {
-    prof::Scope ps(SELM_K_PROJECTION, st);
-    k_dot_part<<<nb, kThreads, 0, st>>>(n, h->cg_x, h->vol, h->part);
-    k_reduce<<<1, kThreads, 0, st>>>(h->part, (int)nb, h->sc + 6);
-    k_sub_scalar<<<eb, kThreads, 0, st>>>(n, h->cg_x, h->sc + 6, 1.0 / h->total_vol);
-    MCK(cudaGetLastError());
-  }
+  MRET(zero_mean(h, st));
   if (iters) *iters = it;
   if (resid) *resid = bn > 0.0 ? rn / bn : 0.0;
   if (bn > 0.0 && rn > tol * bn) {
@@ -1415,6 +1519,11 @@ selm_status selm_mac_create(const selm_mac_desc* desc, void* stream, selm_mac** 
   h->fw2 = (double*)p;
   CREATE_STEP(alloc(h, (size_t)plan.fine_size * 8, &p, st));
   h->fine_buf = (double*)p;
+  if (mac_spectral_supported(d.dim, d.n, d.K) && cudaMalloc(&h->spec, mac_spectral_bytes(d.n, d.K)) == cudaSuccess)
+    h->allocs.push_back(h->spec);
+  else
+    h->spec = nullptr;   // another grid, or no memory for the spectra
+  cudaGetLastError();
   for (double** b : {&h->cg_x, &h->cg_r, &h->cg_z, &h->cg_p, &h->cg_q, &h->pv}) {
     CREATE_STEP(alloc(h, (size_t)nc * 8, &p, st));
     *b = (double*)p;

@@ -1,0 +1,64 @@
+"""The spectral solves behind the staggered composite grid's projection and the
+exact Stokes velocity: every split of rows between the fine and the base part
+(none, one, all but one, all refined), the grid beside them that is not a power
+of two (diagonal preconditioner, FAC), and right-hand sides that are rounding."""
+
+import numpy as np
+import pytest
+import torch
+
+from oracle.composite_mac import CompositeMAC
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def S():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1003_2680_gb300 import selm as mod
+    return mod
+
+
+@pytest.mark.parametrize("n,K", [(4, 0), (4, 1), (4, 4), (8, 7), (16, 3), (12, 4)])
+@pytest.mark.parametrize("adjoint", [0, 1])
+def test_projection(S, n, K, adjoint):
+    """P~ u (or W P~ W^-1 u) against the oracle's direct solve at 1e-11: the
+    pressure to a relative residual of 1e-14, times the operator's condition (a
+    few hundred at these sizes).  Projecting the result again moves it by
+    rounding only, and a zero field stays zero."""
+    g = CompositeMAC(n, K, 3)
+    h = S.selm_mac_create(S.make_mac_desc(3, n, K, projection=1, proj_tol=1e-14))
+    u = np.random.default_rng(n + K).standard_normal(g.n_faces)
+    want = g.weight * g.project(u / g.weight) if adjoint else g.project(u)
+    ud = torch.tensor(u, device="cuda")
+    out = torch.empty_like(ud)
+    S.selm_mac_project(h, ud, out, adjoint=bool(adjoint))
+    got = out.cpu().numpy()
+    assert np.linalg.norm(got - want) <= 1e-11 * np.linalg.norm(want)
+    again = torch.empty_like(out)
+    S.selm_mac_project(h, out, again, adjoint=bool(adjoint))
+    assert ((again - out).norm() / out.norm()).item() <= 1e-11
+    zero = torch.zeros_like(ud)
+    assert S.selm_mac_project(h, zero, out, adjoint=bool(adjoint)) == (0, 0.0)
+    assert not out.any()
+    S.selm_mac_destroy(h)
+
+
+@pytest.mark.parametrize("n", [4, 16, 32, 24])
+def test_stokes_velocity(S, n):
+    """The Stokes velocity of an FP32 handle (spectral, except at 24) against the
+    FP64 handle's FAC solves, both to 1e-11: 1e-9, the tolerance over the Schur
+    complement's smallest eigenvalue."""
+    us = []
+    for prec in (0, 1):
+        h = S.selm_mg_create(S.make_desc(dim=3, n=n, mu=0.9, precision=prec, tol=1e-11))
+        size = S.selm_mg_layout(h, 0, 0, 0)[2]
+        f = torch.tensor(np.random.default_rng(n).standard_normal(size), device="cuda")
+        u = torch.empty_like(f)
+        iters, res = S.selm_mg_stokes_solve(h, f, u)
+        assert res <= 1e-11
+        us.append(u)
+        torch.cuda.synchronize()
+        S.selm_mg_destroy(h)
+    assert ((us[0] - us[1]).norm() / us[0].norm()).item() <= 1e-9
