@@ -51,6 +51,18 @@ __device__ __forceinline__ void normal_of(uint4 w, int lane, double* out) {
   *out = r * ((lane & 1) ? sn : cs);
 }
 
+// The normals of lanes `lane` (0 or 2) and lane + 1: one Box-Muller pair.
+__device__ __forceinline__ void normal_pair(uint4 w, int lane, double* n0, double* n1) {
+  const double s = 2.3283064365386962890625e-10;
+  const uint32_t wa = lane < 2 ? w.x : w.z, wb = lane < 2 ? w.y : w.w;
+  const double ua = ((double)wa + 0.5) * s, ub = ((double)wb + 0.5) * s;
+  const double r = sqrt(-2.0 * log(ua));
+  double sn, cs;
+  sincospi(2.0 * ub, &sn, &cs);
+  *n0 = r * cs;
+  *n1 = r * sn;
+}
+
 // All four Box-Muller normals of one Philox block: u_k = (w_k + 1/2) 2^-32,
 // (n0, n1) = sqrt(-2 ln u0) (cos 2 pi u1, sin 2 pi u1), (n2, n3) likewise.
 template <typename T>

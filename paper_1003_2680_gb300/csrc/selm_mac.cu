@@ -198,7 +198,8 @@ constexpr int kPrefetch = 8;
 template <typename T, int NK, int LANES>
 __global__ void __launch_bounds__(kThreads) k_colour(SellDev S, int pos0, int cnt, T* __restrict__ v,
                                                     const T* __restrict__ b, T sigma, Key key, uint32_t c1,
-                                                    const unsigned long long* __restrict__ cyc) {
+                                                    const unsigned long long* __restrict__ cyc,
+                                                    const T* __restrict__ drawn) {
   pdl_launch_dependents();
   const int g = blockIdx.x * blockDim.x + threadIdx.x;
   const int t = g / LANES, sub = g % LANES;
@@ -226,11 +227,15 @@ __global__ void __launch_bounds__(kThreads) k_colour(SellDev S, int pos0, int cn
     row = S.row[p];
     rd = rd_at<T>(S, p);
     if (NK != 0) {
-      const unsigned long long c = *cyc;
-      const uint32_t id = NK == 1 ? (uint32_t)t : (uint32_t)row;
-      const uint4 wv = philox4x32_10(make_uint4(id >> 2, c1, (uint32_t)c, (uint32_t)(c >> 32)), key.k0, key.k1);
       T gn;
-      normal_of(wv, (int)(id & 3), &gn);
+      if (drawn) {
+        gn = drawn[p];
+      } else {
+        const unsigned long long c = *cyc;
+        const uint32_t id = NK == 1 ? (uint32_t)t : (uint32_t)row;
+        const uint4 wv = philox4x32_10(make_uint4(id >> 2, c1, (uint32_t)c, (uint32_t)(c >> 32)), key.k0, key.k1);
+        normal_of(wv, (int)(id & 3), &gn);
+      }
       ns = sigma * gn;
       rsv = rs_at<T>(S, p);
     }
@@ -251,6 +256,64 @@ __global__ void __launch_bounds__(kThreads) k_colour(SellDev S, int pos0, int cn
   v[row] = nv;
 }
 
+// The normals of every class pass of a FAC cycle, drawn at its start (FP64
+// inner cycles): list position p of a level holds, for each of its sweeps,
+// the normal that the class pass would draw at its row.  In the passes one
+// lane in four of each row draws, and an FP64 instruction takes a warp the
+// same time for 8 active lanes as for 32; here every lane draws, and on the
+// base levels the two normals of a Box-Muller pair (neighbouring ranks) come
+// from one evaluation.
+constexpr int kDrawLists = 16;
+struct DrawList {
+  long long first;             // first thread of the list
+  int npos, sweeps, sweep0;    // list positions, sweeps, index of the first
+  int level1;                  // counter level; slab: 0
+  int slab;                    // 1: normals addressed by the row (kind 2), one per thread
+  int ncol;
+  const int* row;
+  const int* cstart;           // first position of each class
+  double* out;                 // [sweeps][npos]
+};
+struct DrawLists {
+  int n;
+  long long total;
+  DrawList l[kDrawLists];
+};
+
+__global__ void __launch_bounds__(kThreads) k_draw(DrawLists D, Key key, const unsigned long long* __restrict__ cyc) {
+  const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (g >= D.total) return;
+  int q = 0;
+  while (q + 1 < D.n && g >= D.l[q + 1].first) ++q;
+  const DrawList& L = D.l[q];
+  const long long item = g - L.first;
+  const int per = L.slab ? L.npos : L.npos >> 1;   // (classes are padded to whole slices of 32)
+  const int sw = (int)(item / per), p = (int)(item - (long long)sw * per) * (L.slab ? 1 : 2);
+  if (L.row[p] < 0) return;
+  int lo = 0, hi = L.ncol - 1;                     // class of position p
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (L.cstart[mid] <= p)
+      lo = mid;
+    else
+      hi = mid - 1;
+  }
+  const uint32_t id = L.slab ? (uint32_t)L.row[p] : (uint32_t)(p - L.cstart[lo]);
+  const uint32_t c1 = (uint32_t)L.level1 | ((uint32_t)(lo & 15) << 8) | ((uint32_t)(L.sweep0 + sw) << 12) |
+                      ((uint32_t)(L.slab ? 2 : 0) << 20) | ((uint32_t)(lo >> 4) << 24);
+  const unsigned long long c = *cyc;
+  const uint4 w = philox4x32_10(make_uint4(id >> 2, c1, (uint32_t)c, (uint32_t)(c >> 32)), key.k0, key.k1);
+  double* out = L.out + (long long)sw * L.npos + p;
+  if (L.slab) {
+    normal_of(w, (int)(id & 3), out);
+    return;
+  }
+  double a, b;
+  normal_pair(w, (int)(id & 2), &a, &b);
+  out[0] = a;
+  out[1] = b;
+}
+
 // Launch of one class pass with programmatic stream serialisation.  Classes
 // of at least kWideClass rows take one lane per row: a warp then reads each
 // stored entry of its 32 rows as one coalesced access, and a class that large
@@ -259,13 +322,13 @@ constexpr long long kWideClass = 32768;
 
 template <typename T, int NK>
 cudaError_t launch_colour(const SellDev& S, int pos0, int cnt, T* v, const T* b, T sigma, Key key, uint32_t c1,
-                          const unsigned long long* cyc, cudaStream_t st) {
+                          const unsigned long long* cyc, const T* drawn, cudaStream_t st) {
   if (cnt >= kWideClass) {
     const unsigned grid = (unsigned)(((long long)cnt + kThreads - 1) / kThreads);
-    return launch_pdl(k_colour<T, NK, 1>, grid, kThreads, st, S, pos0, cnt, v, b, sigma, key, c1, cyc);
+    return launch_pdl(k_colour<T, NK, 1>, grid, kThreads, st, S, pos0, cnt, v, b, sigma, key, c1, cyc, drawn);
   }
   const unsigned grid = (unsigned)std::max<long long>(1, ((long long)cnt * kRowLanes + kThreads - 1) / kThreads);
-  return launch_pdl(k_colour<T, NK, kRowLanes>, grid, kThreads, st, S, pos0, cnt, v, b, sigma, key, c1, cyc);
+  return launch_pdl(k_colour<T, NK, kRowLanes>, grid, kThreads, st, S, pos0, cnt, v, b, sigma, key, c1, cyc, drawn);
 }
 
 // ---- all colour passes of a small level's sweeps in one thread block --------
@@ -299,7 +362,8 @@ struct RowLane {
 
 template <typename T, int NK>
 __device__ __forceinline__ void row_lane_load(const SellDev& S, int g, int pos0, int cnt, uint32_t c1, T sigma,
-                                              Key key, unsigned long long c64, RowLane<T>& k) {
+                                              Key key, unsigned long long c64, const T* __restrict__ drawn,
+                                              RowLane<T>& k) {
   constexpr int P = BlockPrefetch<T>::value;
   const int t = g / kRowLanes;
   k.sub = g % kRowLanes;
@@ -324,10 +388,14 @@ __device__ __forceinline__ void row_lane_load(const SellDev& S, int g, int pos0,
       k.row = S.row[p];
       k.rd = rd_at<T>(S, p);
       if (NK != 0) {
-        const uint4 wv = philox4x32_10(make_uint4((uint32_t)t >> 2, c1, (uint32_t)c64, (uint32_t)(c64 >> 32)),
-                                       key.k0, key.k1);
         T gn;
-        normal_of(wv, t & 3, &gn);
+        if (drawn) {
+          gn = drawn[p];
+        } else {
+          const uint4 wv = philox4x32_10(make_uint4((uint32_t)t >> 2, c1, (uint32_t)c64, (uint32_t)(c64 >> 32)),
+                                         key.k0, key.k1);
+          normal_of(wv, t & 3, &gn);
+        }
         k.ns = sigma * gn;
         k.rsv = rs_at<T>(S, p);
       }
@@ -371,7 +439,9 @@ __global__ void __launch_bounds__(kBlockSweep) k_colour_block(SellDev S, const i
                                                              const int* __restrict__ csize, int ncol, int level1,
                                                              int sweep0, int nsweeps, int N, T* v,
                                                              const T* __restrict__ b, T sigma, Key key,
-                                                             const unsigned long long* __restrict__ cyc) {
+                                                             const unsigned long long* __restrict__ cyc,
+                                                             const T* __restrict__ drawn) {
+  // drawn: the sweeps' normals one after another, or null
   extern __shared__ __align__(16) unsigned char block_smem[];
   T* vs = reinterpret_cast<T*>(block_smem);
   T* bs = vs + N;
@@ -392,7 +462,7 @@ __global__ void __launch_bounds__(kBlockSweep) k_colour_block(SellDev S, const i
   const int npass = nsweeps * ncol;
   RowLane<T> k;
   if (npass > 0) row_lane_load<T, NK>(S, wbase + (tid & 31), cs[0], cz[0], block_ctr1(level1, 0, sweep0), sigma, key,
-                                      c64, k);
+                                      c64, drawn, k);
   for (int q = 0; q < npass; ++q) {
     const int sw = q / ncol, c = q - sw * ncol;
     const int pos0 = cs[c], cnt = cz[c];
@@ -401,13 +471,14 @@ __global__ void __launch_bounds__(kBlockSweep) k_colour_block(SellDev S, const i
     // classes of more than kBlockSweep / kRowLanes rows: the further lanes
     for (int base = wbase + kBlockSweep; base < cnt * kRowLanes; base += kBlockSweep) {
       RowLane<T> x;
-      row_lane_load<T, NK>(S, base + (tid & 31), pos0, cnt, c1, sigma, key, c64, x);
+      row_lane_load<T, NK>(S, base + (tid & 31), pos0, cnt, c1, sigma, key, c64,
+                           drawn ? drawn + (long long)sw * S.npos : nullptr, x);
       row_lane_apply<T, NK>(S, x, vs, bs);
     }
     if (q + 1 < npass) {   // the next class's static data, before the barrier
       const int sw2 = (q + 1) / ncol, c2 = (q + 1) - sw2 * ncol;
       row_lane_load<T, NK>(S, wbase + (tid & 31), cs[c2], cz[c2], block_ctr1(level1, c2, sweep0 + sw2), sigma, key,
-                           c64, k);
+                           c64, drawn ? drawn + (long long)sw2 * S.npos : nullptr, k);
     }
     __syncthreads();
   }
@@ -747,6 +818,7 @@ struct selm_mac {
     const int* d_cstart = nullptr;
     const int* d_csize = nullptr;
     bool block_sweeps = false;
+    double* drawn = nullptr;         // normals of its sweeps (FP64 inner cycles)
   };
   std::vector<Level> lev;
   const double* Linv = nullptr;
@@ -761,6 +833,8 @@ struct selm_mac {
   SellDev E;
   LevelDev fine{};                   // the uniform fine lattice of the particle kernel
   long long fine_size = 0;
+  DrawLists draws{};                 // what k_draw fills at the start of a noisy cycle (n = 0: drawn at the rows)
+  double* drawn_patch = nullptr;
   // buffers
   void *r = nullptr, *q = nullptr;   // composite residual / correction (inner precision)
   double* xi = nullptr;
@@ -869,6 +943,13 @@ uint32_t ctr1(int level, int comp, int colour, int sweep, int kind) {
          ((uint32_t)kind << 20) | ((uint32_t)(colour >> 4) << 24);
 }
 
+// Normals of sweep s of a list (null: drawn at the rows).
+template <typename T>
+const T* drawn_at(const double* base, int npos, int s) {
+  if constexpr (sizeof(T) == 8) return base ? base + (long long)s * npos : nullptr;
+  return nullptr;
+}
+
 // ---- the V-cycle on the base hierarchy (Algorithm 3) -------------------------
 template <typename T>
 selm_status sweep(selm_mac* h, int l, int s, double sigma, const unsigned long long* cyc, cudaStream_t st) {
@@ -878,9 +959,9 @@ selm_status sweep(selm_mac* h, int l, int s, double sigma, const unsigned long l
     prof::Scope ps(SELM_K_COARSE_SWEEP, st);
     if (sigma != 0.0)
       MCK((launch_colour<T, 1>(L.cls, L.cstart[c], cnt, (T*)L.v, (const T*)L.b, (T)sigma, h->key,
-                              ctr1(l + 1, 0, (int)c, s, 0), cyc, st)));
+                              ctr1(l + 1, 0, (int)c, s, 0), cyc, drawn_at<T>(L.drawn, L.cls.npos, s), st)));
     else
-      MCK((launch_colour<T, 0>(L.cls, L.cstart[c], cnt, (T*)L.v, (const T*)L.b, (T)0, h->key, 0, cyc, st)));
+      MCK((launch_colour<T, 0>(L.cls, L.cstart[c], cnt, (T*)L.v, (const T*)L.b, (T)0, h->key, 0, cyc, nullptr, st)));
   }
   return SELM_OK;
 }
@@ -900,10 +981,11 @@ selm_status sweeps(selm_mac* h, int l, int s0, int n, double sigma, const unsign
   const size_t smem = block_sweep_smem<T>(L.N, ncol);
   if (sigma != 0.0)
     k_colour_block<T, 1><<<1, kBlockSweep, smem, st>>>(L.cls, L.d_cstart, L.d_csize, ncol, l + 1, s0, n, (int)L.N,
-                                                       (T*)L.v, (const T*)L.b, (T)sigma, h->key, cyc);
+                                                       (T*)L.v, (const T*)L.b, (T)sigma, h->key, cyc,
+                                                       drawn_at<T>(L.drawn, L.cls.npos, s0));
   else
     k_colour_block<T, 0><<<1, kBlockSweep, smem, st>>>(L.cls, L.d_cstart, L.d_csize, ncol, l + 1, s0, n, (int)L.N,
-                                                       (T*)L.v, (const T*)L.b, (T)0, h->key, cyc);
+                                                       (T*)L.v, (const T*)L.b, (T)0, h->key, cyc, nullptr);
   MCK(cudaGetLastError());
   return SELM_OK;
 }
@@ -946,6 +1028,11 @@ selm_status vcycle(selm_mac* h, int l, double sigma, const unsigned long long* c
 template <typename T>
 selm_status correction(selm_mac* h, double sigma, const unsigned long long* cyc, cudaStream_t st) {
   selm_mac::Level& B = h->lev[0];
+  if (sigma != 0.0 && h->draws.n > 0) {
+    prof::Scope ps(SELM_K_OTHER, st);
+    k_draw<<<blocks_for(h->draws.total), kThreads, 0, st>>>(h->draws, h->key, cyc);
+    MCK(cudaGetLastError());
+  }
   {
     prof::Scope ps(SELM_K_RESTRICT, st);
     MCK((launch_pdl(k_sell_mv<T, 0>, blocks_for(h->Pt.npos), kThreads, st, h->Pt, (const T*)h->r, (T*)B.b, nullptr)));
@@ -962,9 +1049,10 @@ selm_status correction(selm_mac* h, double sigma, const unsigned long long* cyc,
       prof::Scope ps(SELM_K_FINE_SWEEP, st);
       if (sigma != 0.0)
         MCK((launch_colour<T, 2>(h->Apatch, h->pstart[c], cnt, (T*)h->q, (const T*)h->r, (T)sigma, h->key,
-                                ctr1(0, 0, (int)c, s, 2), cyc, st)));
+                                ctr1(0, 0, (int)c, s, 2), cyc, drawn_at<T>(h->drawn_patch, h->Apatch.npos, s), st)));
       else
-        MCK((launch_colour<T, 0>(h->Apatch, h->pstart[c], cnt, (T*)h->q, (const T*)h->r, (T)0, h->key, 0, cyc, st)));
+        MCK((launch_colour<T, 0>(h->Apatch, h->pstart[c], cnt, (T*)h->q, (const T*)h->r, (T)0, h->key, 0, cyc, nullptr,
+                                st)));
     }
   return SELM_OK;
 }
@@ -1489,6 +1577,37 @@ selm_status selm_mac_create(const selm_mac_desc* desc, void* stream, selm_mac** 
       Et.ptr[rr + 1] = (long long)Et.col.size();
     }
     CREATE_STEP(upload_sell(h, make_sell(Et, natural_order(Et.nr), false), false, &h->Et, st));
+  }
+  if (!f32 && plan.levels < kDrawLists) {   // buffers of the normals; without memory for them the rows draw
+    long long normals = 0;
+    for (int l = 0; l + 1 < plan.levels; ++l) normals += (long long)h->lev[l].cls.npos * (d.nu_pre + d.nu_post);
+    if (!h->pstart.empty()) normals += (long long)h->Apatch.npos * d.nu_patch;
+    double* base = nullptr;
+    if (normals > 0 && cudaMalloc((void**)&base, normals * sizeof(double)) == cudaSuccess) {
+      h->allocs.push_back(base);
+      auto add = [&](const SellDev& S, const std::vector<int>& starts, int sweeps, int level1, bool slab,
+                     double** out) -> selm_status {
+        if (sweeps <= 0) return SELM_OK;
+        DrawList& q = h->draws.l[h->draws.n++];
+        q.first = h->draws.total;
+        q.npos = S.npos;
+        q.sweeps = sweeps;
+        q.sweep0 = 0;
+        q.level1 = level1;
+        q.slab = slab ? 1 : 0;
+        q.ncol = (int)starts.size();
+        q.row = S.row;
+        q.out = base;
+        *out = base;
+        base += (long long)S.npos * sweeps;
+        h->draws.total += (long long)sweeps * (slab ? S.npos : S.npos / 2);
+        return upload(h, starts, &q.cstart, st);
+      };
+      for (int l = 0; l + 1 < plan.levels; ++l)
+        CREATE_STEP(add(h->lev[l].cls, h->lev[l].cstart, d.nu_pre + d.nu_post, l + 1, false, &h->lev[l].drawn));
+      if (!h->pstart.empty()) CREATE_STEP(add(h->Apatch, h->pstart, d.nu_patch, 0, true, &h->drawn_patch));
+    }
+    cudaGetLastError();
   }
   // the uniform fine lattice of the particle kernel
   h->fine.level = 0;
