@@ -287,9 +287,18 @@ selm_status vcycle_t(selm_mg* h, Sys& s, int l, T* v0, const T* b0, bool noise, 
   // A level above the engine with at most 2^20 sites per component: each half
   // of its V-cycle in one cooperative launch (one or a few site updates per
   // thread per pass).  Larger levels keep one GPU-wide launch per colour pass,
-  // whose parallelism then beats the launch overhead.
-  if (l > 0 && !last && !L.rb && level_sites(L) <= kCoopMaxSites && s.use_engine && s.use_coop && eng.valid && l < eng.params.l0 &&
-      s.coop_bar && level_coop_supported<T>(L)) {
+  // whose parallelism then beats the launch overhead.  In dataflow order that
+  // already holds for 3-D levels of more than a million unknowns: a pass costs
+  // about 3 us of update latency plus its sites over 78 K threads, a launch per
+  // pass less once it is full (V-cycle with level 1 of 64^3 446 us cooperative,
+  // 527 per pass; 72^3: 831 and 757; 96^3: 1236 and 1076).  Those passes store the
+  // same parity bits, so both forms give the same values.
+  const bool flow_level = sizeof(T) == 4 && s.coop_flow && L.flow;
+  const bool full_passes = flow_level && L.c[0].ny > 1 && L.size > 1000000 && coarse_rows8(L);
+  const bool coop = l > 0 && !last && !L.rb && level_sites(L) <= kCoopMaxSites && s.use_engine && s.use_coop &&
+                    eng.valid && l < eng.params.l0 && s.coop_bar && level_coop_supported<T>(L);
+  const bool tags = coop && full_passes;
+  if (coop && !full_passes) {
     const LevelDev& Lc = s.lev[l + 1];
     CK(launch_level_coop<T>(L, Lc, 0, h->mu1, h->mu2, v, b, (T*)s.t[l], (T*)s.b[l + 1], (T*)s.v[l + 1], s.coop_bar,
                             s.coop_flow, noise, h->key, cyc, st));
@@ -308,7 +317,7 @@ selm_status vcycle_t(selm_mg* h, Sys& s, int l, T* v0, const T* b0, bool noise, 
     CK(launch_coarsest<T>(L, v, b, noise, h->key, cyc, st));
     return SELM_OK;
   }
-  for (int q = 0; q < h->mu1; ++q) CK(launch_smooth<T>(L, v, b, q, noise, h->key, cyc, st));
+  for (int q = 0; q < h->mu1; ++q) CK(launch_smooth<T>(L, v, b, q, noise, h->key, cyc, st, tags ? (q + 1) & 1 : -1));
   if (!last) {
     const LevelDev& Lc = s.lev[l + 1];
     CK(launch_residual<T>(L, v, b, (T*)s.t[l], st));
@@ -317,9 +326,10 @@ selm_status vcycle_t(selm_mg* h, Sys& s, int l, T* v0, const T* b0, bool noise, 
       CK(cudaMemsetAsync(s.v[l + 1], 0, (size_t)Lc.size * sizeof(T), st));
     selm_status r = vcycle_t<T>(h, s, l + 1, v0, b0, noise, cyc, st);
     if (r != SELM_OK) return r;
-    CK(launch_prolong<T>(L, Lc, v, (const T*)s.v[l + 1], st));
+    CK(launch_prolong<T>(L, Lc, v, (const T*)s.v[l + 1], st, tags));
   }
-  for (int q = 0; q < h->mu2; ++q) CK(launch_smooth<T>(L, v, b, h->mu1 + q, noise, h->key, cyc, st));
+  for (int q = 0; q < h->mu2; ++q)
+    CK(launch_smooth<T>(L, v, b, h->mu1 + q, noise, h->key, cyc, st, tags ? (q + 1) & 1 : -1));
   return SELM_OK;
 }
 

@@ -743,6 +743,14 @@ __device__ __forceinline__ void galerkin_residual_seg(const CompDev& c, const T*
   }
 }
 
+// The value an update stores when the level's passes carry the parity of the
+// update count in the last mantissa bit (see the dataflow order below): tag 0
+// or 1; tag < 0: the value itself.
+__device__ __forceinline__ float tagged(float v, int tag) {
+  return tag < 0 ? v : __uint_as_float((__float_as_uint(v) & ~1u) | (unsigned)tag);
+}
+__device__ __forceinline__ double tagged(double v, int) { return v; }
+
 // Heat-bath update of site g of a Galerkin colour pass (g runs over the
 // class sites of all components, component ci from cp.gstart):
 // v_i = (b_i - sum_{j != i} A_ij v_j) / A_ii + n / sqrt(A_ii).  The four
@@ -1215,7 +1223,7 @@ __global__ void __launch_bounds__(kBlock) k_coarse_site(LevelDev L, ColourPass c
 template <typename T, bool NOISE, int CX, bool CG>
 __device__ __forceinline__ void coarse_colour_v8_item(const LevelDev& L, const ColourPass& cp, const ColumnPass& sp,
                                                       T* __restrict__ v, const T* __restrict__ b, int sweep, Key key,
-                                                      unsigned long long cy, long long g) {
+                                                      unsigned long long cy, long long g, int tag = -1) {
   if (g >= sp.start[L.ncomp]) return;
   int ci = 0;
   while (ci + 1 < L.ncomp && g >= sp.start[ci + 1]) ++ci;
@@ -1292,18 +1300,19 @@ __device__ __forceinline__ void coarse_colour_v8_item(const LevelDev& L, const C
   for (int e = 0; e < 4; ++e) {
     T nv = ((CG ? __ldcg(b + rowi + 2 * e) : LdNC::ld(b + rowi + 2 * e)) - acc[e]) / diag;
     if (NOISE) nv += n4[e] / tsqrt(diag);
-    v[rowi + 2 * e] = nv;
+    v[rowi + 2 * e] = tagged(nv, tag);
   }
 }
 
 template <typename T, bool NOISE, int CX>
 __global__ void __launch_bounds__(kBlock) k_coarse_colour_v8(LevelDev L, ColourPass cp, ColumnPass sp,
                                                             T* __restrict__ v, const T* __restrict__ b, int sweep,
-                                                            Key key, const unsigned long long* __restrict__ cyc) {
+                                                            Key key, const unsigned long long* __restrict__ cyc,
+                                                            int tag) {
   pdl_enter();
   const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (g >= sp.start[L.ncomp]) return;
-  coarse_colour_v8_item<T, NOISE, CX, false>(L, cp, sp, v, b, sweep, key, NOISE ? *cyc : 0ull, g);
+  coarse_colour_v8_item<T, NOISE, CX, false>(L, cp, sp, v, b, sweep, key, NOISE ? *cyc : 0ull, g, tag);
 }
 
 // ---------------------------------------------------------------------------
@@ -1608,11 +1617,11 @@ __device__ __forceinline__ void prolong_seg8(const LevelDev& Lf, const LevelDev&
   Vec<T>::store8(out, cur);
 }
 
-template <typename T>
+template <typename T, bool TAG0>
 __global__ void __launch_bounds__(kBlock) k_prolong_v8(LevelDev Lf, LevelDev Lc, RowPass rp, T* __restrict__ v,
                                                       const T* __restrict__ vc) {
   pdl_enter();
-  prolong_seg8<T, false>(Lf, Lc, rp, v, vc, (long long)blockIdx.x * blockDim.x + threadIdx.x);
+  prolong_seg8<T, TAG0>(Lf, Lc, rp, v, vc, (long long)blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -3087,9 +3096,16 @@ long long column_pass(const LevelDev& L, int log2w, ColumnPass* cp) {
   return items;
 }
 
+// 8-wide rows, x modulus 2: four class sites (one noise group) per thread.
+bool coarse_rows8(const LevelDev& L) {
+  for (int ci = 0; ci < L.ncomp; ++ci)
+    if (L.c[ci].nx % 8 != 0 || L.c[ci].mx != 2) return false;
+  return true;
+}
+
 template <typename T>
 cudaError_t launch_smooth(const LevelDev& L, T* v, const T* b, int sweep, bool noise, Key key,
-                          const unsigned long long* cyc, cudaStream_t st) {
+                          const unsigned long long* cyc, cudaStream_t st, int tag) {
   if (L.level == 0 && L.c[0].nx % 8 == 0) {
     ColumnPass cp{};
     const long long items = column_pass<T>(L, 3, &cp);
@@ -3153,9 +3169,8 @@ cudaError_t launch_smooth(const LevelDev& L, T* v, const T* b, int sweep, bool n
   }
   int maxcol = 0;
   for (int ci = 0; ci < L.ncomp; ++ci) maxcol = maxcol > L.c[ci].ncol ? maxcol : L.c[ci].ncol;
-  bool v8 = true;   // 8-wide rows, x modulus 2: four class sites (one noise group) per thread
-  for (int ci = 0; ci < L.ncomp; ++ci)
-    if (L.c[ci].nx % 8 != 0 || L.c[ci].mx != 2) v8 = false;
+  const bool v8 = coarse_rows8(L);
+  if (tag >= 0 && !v8) return cudaErrorNotSupported;
   for (int q = 0; q < maxcol; ++q) {
     ColourPass cp{};
     const long long gs = colour_pass_of(L, q, &cp);
@@ -3171,13 +3186,17 @@ cudaError_t launch_smooth(const LevelDev& L, T* v, const T* b, int sweep, bool n
       sp.start[L.ncomp] = items;
       const int cx = q % 2;   // every component has x modulus 2
       if (noise && cx == 0)
-        LTRY(launch_pdl(k_coarse_colour_v8<T, true, 0>, grid_for(items), kBlock, st, L, cp, sp, v, b, sweep, key, cyc));
+        LTRY(launch_pdl(k_coarse_colour_v8<T, true, 0>, grid_for(items), kBlock, st, L, cp, sp, v, b, sweep, key, cyc,
+                        tag));
       else if (noise)
-        LTRY(launch_pdl(k_coarse_colour_v8<T, true, 1>, grid_for(items), kBlock, st, L, cp, sp, v, b, sweep, key, cyc));
+        LTRY(launch_pdl(k_coarse_colour_v8<T, true, 1>, grid_for(items), kBlock, st, L, cp, sp, v, b, sweep, key, cyc,
+                        tag));
       else if (cx == 0)
-        LTRY(launch_pdl(k_coarse_colour_v8<T, false, 0>, grid_for(items), kBlock, st, L, cp, sp, v, b, sweep, key, cyc));
+        LTRY(launch_pdl(k_coarse_colour_v8<T, false, 0>, grid_for(items), kBlock, st, L, cp, sp, v, b, sweep, key, cyc,
+                        tag));
       else
-        LTRY(launch_pdl(k_coarse_colour_v8<T, false, 1>, grid_for(items), kBlock, st, L, cp, sp, v, b, sweep, key, cyc));
+        LTRY(launch_pdl(k_coarse_colour_v8<T, false, 1>, grid_for(items), kBlock, st, L, cp, sp, v, b, sweep, key, cyc,
+                        tag));
       continue;
     }
     if (noise)
@@ -3244,7 +3263,7 @@ cudaError_t launch_restrict(const LevelDev& Lf, const LevelDev& Lc, const T* t, 
 }
 
 template <typename T>
-cudaError_t launch_prolong(const LevelDev& Lf, const LevelDev& Lc, T* v, const T* vc, cudaStream_t st) {
+cudaError_t launch_prolong(const LevelDev& Lf, const LevelDev& Lc, T* v, const T* vc, cudaStream_t st, bool tag0) {
   prof::Scope ps(SELM_K_PROLONG, st);
   if (Lf.c[0].nx % 8 == 0) {
     RowPass rp{};
@@ -3254,7 +3273,11 @@ cudaError_t launch_prolong(const LevelDev& Lf, const LevelDev& Lc, T* v, const T
       rows += Lf.c[ci].ny * Lf.c[ci].nz;
     }
     rp.rstart[Lf.ncomp] = rows;
-    LTRY(launch_pdl(k_prolong_v8<T>, grid_for((long long)rows * (Lf.c[0].nx >> 3)), kBlock, st, Lf, Lc, rp, v, vc));
+    const unsigned grid = grid_for((long long)rows * (Lf.c[0].nx >> 3));
+    if (tag0)
+      LTRY(launch_pdl(k_prolong_v8<T, true>, grid, kBlock, st, Lf, Lc, rp, v, vc));
+    else
+      LTRY(launch_pdl(k_prolong_v8<T, false>, grid, kBlock, st, Lf, Lc, rp, v, vc));
     return cudaGetLastError();
   }
   k_prolong<T><<<grid_for(Lf.size), kBlock, 0, st>>>(Lf, Lc, v, vc);
@@ -3506,10 +3529,10 @@ cudaError_t launch_philox(const uint32_t* ctr, Key key, uint32_t* out, int n, cu
 
 #define SELM_INSTANTIATE(T)                                                                                  \
   template cudaError_t launch_smooth<T>(const LevelDev&, T*, const T*, int, bool, Key,                      \
-                                        const unsigned long long*, cudaStream_t);                           \
+                                        const unsigned long long*, cudaStream_t, int);                      \
   template cudaError_t launch_residual<T>(const LevelDev&, const T*, const T*, T*, cudaStream_t);           \
   template cudaError_t launch_restrict<T>(const LevelDev&, const LevelDev&, const T*, T*, cudaStream_t);    \
-  template cudaError_t launch_prolong<T>(const LevelDev&, const LevelDev&, T*, const T*, cudaStream_t);     \
+  template cudaError_t launch_prolong<T>(const LevelDev&, const LevelDev&, T*, const T*, cudaStream_t, bool);  \
   template bool level_coop_supported<T>(const LevelDev&);                                                   \
   template cudaError_t launch_level_coop<T>(const LevelDev&, const LevelDev&, int, int, int, T*, const T*, T*, T*, \
                                             T*, unsigned*, bool, bool, Key, const unsigned long long*,            \

@@ -48,9 +48,13 @@ inline int z_chunk(long long cols, int nz, int esize) {
 // Stage kernels.  `T` is float or double (inner precision); all launches go
 // on `st`.  Counters (`cyc`) are read from device memory so that the calls can
 // be captured in CUDA graphs.
+// launch_smooth's tag (Galerkin levels with coarse_rows8()): 0 or 1, the parity
+// bit that FP32 updates store in dataflow order (launch_level_coop); -1: none.
+// launch_prolong's tag0 clears the bit (update count 0).
+bool coarse_rows8(const LevelDev& L);
 template <typename T>
 cudaError_t launch_smooth(const LevelDev& L, T* v, const T* b, int sweep, bool noise, Key key,
-                          const unsigned long long* cyc, cudaStream_t st);
+                          const unsigned long long* cyc, cudaStream_t st, int tag = -1);
 template <typename T>
 cudaError_t launch_residual(const LevelDev& L, const T* v, const T* b, T* t, cudaStream_t st);
 template <typename T>
@@ -58,7 +62,7 @@ cudaError_t launch_restrict(const LevelDev& Lf, const LevelDev& Lc, const T* t, 
                             cudaStream_t st);
 template <typename T>
 cudaError_t launch_prolong(const LevelDev& Lf, const LevelDev& Lc, T* v, const T* vc,
-                           cudaStream_t st);
+                           cudaStream_t st, bool tag0 = false);
 // One Galerkin level (L.level >= 1) as a single cooperative launch over the
 // GPU.  phase 0: the descending half of the V-cycle at this level (mu1
 // sweeps from the zero start in v, residual into t, restriction into bc,

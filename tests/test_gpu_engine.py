@@ -34,3 +34,24 @@ def test_uneven_vcycle(dim, n, prec, mode):
     multigrid.vcycle(osys, 0, want, b0, philox.PhiloxNoise(11, 3, 7), 1.0,
                      coarse_mode="smooth" if mode else "cholesky")
     assert rel(from_dev(m.h, v), want) < tol
+
+
+@pytest.mark.parametrize("noise", [0, 1])
+def test_full_passes_keep_dataflow_values(noise):
+    """Level 1 of 72^3 (144^3 grid): one launch per colour pass with the dataflow
+    order's parity bits, against the plain per-pass form: every stored value
+    within an ulp, so the V-cycles agree to the FP32 tolerance."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1003_2680_gb300 import selm as S
+    m = S.SelmMG(dim=3, n=144, precision=1, seed=11, instance=3)
+    size = m.layout()[1]
+    b = torch.randn(size, device="cuda", generator=torch.Generator("cuda").manual_seed(5))
+    out = []
+    for coop in (1, 0):
+        S.selm_mg_set_option(m.h, S.SELM_OPT_LEVEL_COOP, coop)
+        v = torch.zeros_like(b)
+        S.selm_mg_vcycle(m.h, 0, v, b, 7, noise)
+        out.append(v)
+    assert ((out[0] - out[1]).norm() / out[1].norm()).item() < 1e-5
+    assert not torch.equal(out[0], out[1])
