@@ -28,6 +28,7 @@
 #include <cuda_runtime.h>
 
 #include <cmath>
+#include <cstdint>
 #include <cstdio>
 #include <new>
 #include <string>
@@ -427,6 +428,23 @@ struct DF {
 
 __device__ __forceinline__ DF df_from(float h, float l) { return {h, l}; }
 
+template <int W>
+__device__ __forceinline__ void ld_vec(const float* p, float x[W]) {
+  if constexpr (W == 4) {
+    const float4 q = *reinterpret_cast<const float4*>(p);
+    x[0] = q.x, x[1] = q.y, x[2] = q.z, x[3] = q.w;
+  } else {
+    x[0] = *p;
+  }
+}
+template <int W>
+__device__ __forceinline__ void st_vec(float* p, const float x[W]) {
+  if constexpr (W == 4)
+    *reinterpret_cast<float4*>(p) = make_float4(x[0], x[1], x[2], x[3]);
+  else
+    *p = x[0];
+}
+
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
   s = __fadd_rn(a, b);
   const float bb = __fsub_rn(s, a);
@@ -721,33 +739,62 @@ __global__ void __launch_bounds__(kCBlock) k_comp_residual_df_base(CompGeo G, co
   Vec<float>::store8(rb + c * G.bsize + rbase + x0, out);
 }
 
-// z += q for the double-float chain (covered base rows untouched).
+// z += q for the double-float chain (covered base rows untouched), and the
+// chain's FP64 copy (covered base rows 0).  Both stream the whole chain once, W
+// values per thread: W = 4 where every base plane and so every part's start is a
+// multiple of four, else 1.  At 256^3 with a 256^3 patch (111 M values) the
+// update takes 261 us with W = 4 (408 with W = 1: a 64-bit remainder and
+// 4-byte accesses per value), the copy 230 us with the FP32 values widened
+// by integer operations (542 by conversion instructions, which share GB300's
+// narrow FP64 pipe with the add).
+template <int W>
 __global__ void __launch_bounds__(kCBlock) k_comp_update_df(CompGeo G, float* __restrict__ zh, float* __restrict__ zl,
                                                             const float* __restrict__ vp, const float* __restrict__ vb) {
-  const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  float q;
+  const long long s = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * W;
+  const float* src;
   if (s < G.N0) {
-    q = vp[s];
+    src = vp + s;
   } else if (s < G.N0 + G.N1) {
-    const long long s1 = s - G.N0;
-    if ((int)((s1 % G.bsize) / ((long long)G.bx * G.by)) < G.K) return;
-    q = vb[s1];
+    const long long s1 = s - G.N0, covered = (long long)G.K * G.bx * G.by;
+    for (int c = 0; c < G.ncomp; ++c)
+      if (s1 >= c * G.bsize && s1 - c * G.bsize < covered) return;
+    src = vb + s1;
   } else {
     return;
   }
-  float a, e;
-  two_sum(zh[s], q, a, e);
-  const DF r = df_norm(a, __fadd_rn(e, zl[s]));
-  zh[s] = r.h;
-  zl[s] = r.l;
+  float q[W], h[W], l[W];
+  ld_vec<W>(src, q);
+  ld_vec<W>(zh + s, h);
+  ld_vec<W>(zl + s, l);
+#pragma unroll
+  for (int e = 0; e < W; ++e) {
+    float a, r;
+    two_sum(h[e], q[e], a, r);
+    const DF d = df_norm(a, __fadd_rn(r, l[e]));
+    h[e] = d.h;
+    l[e] = d.l;
+  }
+  st_vec<W>(zh + s, h);
+  st_vec<W>(zl + s, l);
 }
 
-// FP64 copy of the double-float chain (covered base rows 0).
+template <int W>
 __global__ void __launch_bounds__(kCBlock) k_comp_df_to_f64(CompGeo G, const float* __restrict__ zh,
                                                             const float* __restrict__ zl, double* __restrict__ out) {
-  const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const long long s = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * W;
   if (s >= G.N0 + G.N1) return;
-  out[s] = (double)zh[s] + (double)zl[s];
+  float h[W], l[W];
+  ld_vec<W>(zh + s, h);
+  ld_vec<W>(zl + s, l);
+  double o[W];
+#pragma unroll
+  for (int e = 0; e < W; ++e) o[e] = fx_widen(h[e]) + fx_widen(l[e]);
+  if constexpr (W == 4) {
+    reinterpret_cast<double2*>(out + s)[0] = make_double2(o[0], o[1]);
+    reinterpret_cast<double2*>(out + s)[1] = make_double2(o[2], o[3]);
+  } else {
+    out[s] = o[0];
+  }
 }
 
 // Main pass (late = 0) of a patch sweep marching along the patch layers: one
@@ -1058,6 +1105,10 @@ selm_status patch_sweeps_t(selm_comp* C, T* vp, const T* vb, const T* rp, int co
   return SELM_OK;
 }
 
+// Every plane of the base, and with them every component and both parts, start at a
+// multiple of four values (patch planes: one or four times a base plane).
+bool df_quads(const CompGeo& G) { return (long long)G.bx * G.by % 4 == 0 && G.N0 % 4 == 0; }
+
 // The correction half of one FAC iteration, after residual_t filled the
 // level-0 and level-1 b fields from z: restrict, base V-cycle, prolong, patch
 // sweeps, z += q.
@@ -1092,9 +1143,12 @@ selm_status correct_t(selm_comp* C, double* z, bool noise, const unsigned long l
   if (r != SELM_OK) return r;
   {
     prof::Scope ps(SELM_K_OUTER_UPDATE, st);
-    if (zh)
-      k_comp_update_df<<<cgrid(G.N0 + G.N1), kCBlock, 0, st>>>(G, zh, zl, (const float*)s.v[0],
-                                                               (const float*)s.v[1]);
+    if (zh && df_quads(G))
+      k_comp_update_df<4><<<cgrid((G.N0 + G.N1) / 4), kCBlock, 0, st>>>(G, zh, zl, (const float*)s.v[0],
+                                                                        (const float*)s.v[1]);
+    else if (zh)
+      k_comp_update_df<1><<<cgrid(G.N0 + G.N1), kCBlock, 0, st>>>(G, zh, zl, (const float*)s.v[0],
+                                                                  (const float*)s.v[1]);
     else
       k_comp_update<T><<<cgrid(G.N0 + G.N1), kCBlock, 0, st>>>(G, z, (const T*)s.v[0], (const T*)s.v[1]);
   }
@@ -1371,7 +1425,11 @@ selm_status selm_comp_sample(selm_comp* C, int ncycles, double* xi_out, void* st
   if (xi_out) {
     if (C->xh) {
       prof::Scope ps(SELM_K_OTHER, st);
-      k_comp_df_to_f64<<<cgrid(C->geo.N0 + C->geo.N1), kCBlock, 0, st>>>(C->geo, C->xh, C->xl, xi_out);
+      const CompGeo& G = C->geo;
+      if (df_quads(G) && ((uintptr_t)xi_out & 15) == 0)
+        k_comp_df_to_f64<4><<<cgrid((G.N0 + G.N1) / 4), kCBlock, 0, st>>>(G, C->xh, C->xl, xi_out);
+      else
+        k_comp_df_to_f64<1><<<cgrid(G.N0 + G.N1), kCBlock, 0, st>>>(G, C->xh, C->xl, xi_out);
       CCK(cudaGetLastError());
     } else {
       CCK(cudaMemcpyAsync(xi_out, C->xi, (size_t)(C->geo.N0 + C->geo.N1) * sizeof(double), cudaMemcpyDeviceToDevice,

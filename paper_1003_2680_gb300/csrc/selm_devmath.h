@@ -204,4 +204,16 @@ __device__ __forceinline__ void colour_update(T cen[8], const T bb[8], const Col
   }
 }
 
+// FP32 -> FP64 (exact) without the conversion instruction, which runs on
+// GB300's narrow FP64 pipe: the exponent is re-biased by integer operations, a
+// subnormal first scaled by 2^64 in FP32 (exact).
+__device__ __forceinline__ double fx_widen(float f) {
+  const bool sub = (__float_as_uint(f) & 0x7f800000u) == 0u;
+  const unsigned u = __float_as_uint(sub ? f * 18446744073709551616.0f : f);
+  const unsigned ex = (u >> 23) & 0xffu;
+  const unsigned dx = ex == 0u ? 0u : ex == 0xffu ? 0x7ffu : ex + (sub ? 832u : 896u);   // +1023 - 127 (- 64)
+  return __hiloint2double((int)((u & 0x80000000u) | (dx << 20) | ((u & 0x7fffffu) >> 3)), (int)(u << 29));
+}
+__device__ __forceinline__ double fx_widen(double f) { return f; }
+
 }  // namespace selm

@@ -505,18 +505,6 @@ __global__ void __launch_bounds__(kBlock) k_outer_residual_fx(LevelDev L, RowPas
   }
 }
 
-// FP32 -> FP64 (exact) by integer operations for normal values; zero,
-// subnormal and non-finite values through the conversion instruction.
-__device__ __forceinline__ double fx_widen(float f) {
-  const unsigned u = __float_as_uint(f);
-  const unsigned ex = (u >> 23) & 0xffu;
-  if (ex == 0u || ex == 0xffu) return (double)f;
-  return __longlong_as_double((long long)(((unsigned long long)(u & 0x80000000u) << 32) |
-                                          ((unsigned long long)(ex - 127u + 1023u) << 52) |
-                                          ((unsigned long long)(u & 0x7fffffu) << 29)));
-}
-__device__ __forceinline__ double fx_widen(double f) { return f; }
-
 // z += d: one FP64 add per unknown (the widening of an FP32 d is done by
 // integer operations, off GB300's narrow FP64 pipe).
 template <typename T>

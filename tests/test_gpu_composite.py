@@ -289,3 +289,33 @@ def test_bench_size_fac_cycle_is_translation_equivariant(S):
     ds = zs - _roll(S, c, z0, 192)
     assert (torch.linalg.vector_norm(ds - d) / torch.linalg.vector_norm(d)).item() < 1e-5
     S.selm_comp_destroy(c)
+
+
+@pytest.mark.parametrize("dim,n,K", [(2, 64, 4), (3, 32, 4)])
+def test_chain_copy_alignment(S, dim, n, K):
+    """The FP64 copy of a double-float chain into 16- and 8-byte aligned buffers
+    (four values and one value per thread): the same values."""
+    buf = []
+    for shift in (0, 1):
+        c, _ = handle(S, dim, n, K, "fp32", seed=9, instance=4)
+        raw = torch.zeros(S.selm_comp_size(c) + 2, dtype=torch.float64, device="cuda")
+        S.selm_comp_sample(c, 2, raw[shift:])
+        buf.append(raw[shift:shift + S.selm_comp_size(c)])
+        assert raw[S.selm_comp_size(c) + shift].item() == 0.0
+    assert torch.equal(buf[0], buf[1])
+
+
+def test_outer_update_widens_exactly(S):
+    """FP32 corrections of every exponent class (zeros, subnormals, normals,
+    infinities) added to z = 0: FP64 holds each exactly."""
+    from paper_1003_2680_gb300 import selm
+    m = selm.SelmMG(dim=2, n=64, precision=1, seed=1, instance=0)
+    size = selm.selm_mg_layout(m.h, 0, 0, 0)[2]
+    bits = torch.randint(-2**31, 2**31 - 1, (size,), dtype=torch.int64, generator=torch.Generator().manual_seed(3))
+    bits[:512] &= 0x807fffff
+    bits[512:516] = torch.tensor([0, -2**31, 0x7f800000, 0xff800000 - 2**32])
+    d = bits.to(torch.int32).view(torch.float32)
+    d = torch.where(torch.isnan(d), torch.ones_like(d), d).cuda()
+    z = torch.zeros(size, dtype=torch.float64, device="cuda")
+    selm.selm_mg_outer_update(m.h, 0, z, d)
+    assert torch.equal(z, d.double())

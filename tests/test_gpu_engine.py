@@ -9,7 +9,7 @@ import torch
 
 import selm_inputs
 from oracle import grid, multigrid, philox
-from tests.gpu_util import from_dev, rel, round_like, to_dev
+from tests.gpu_util import comps, from_dev, rel, round_like, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -45,8 +45,7 @@ def test_full_passes_keep_dataflow_values(noise):
         pytest.skip("no CUDA device")
     from paper_1003_2680_gb300 import selm as S
     m = S.SelmMG(dim=3, n=144, precision=1, seed=11, instance=3)
-    size = m.layout()[1]
-    b = torch.randn(size, device="cuda", generator=torch.Generator("cuda").manual_seed(5))
+    b = torch.randn(comps(m.h, 0, 0)[1], device="cuda", generator=torch.Generator("cuda").manual_seed(5))
     out = []
     for coop in (1, 0):
         S.selm_mg_set_option(m.h, S.SELM_OPT_LEVEL_COOP, coop)
