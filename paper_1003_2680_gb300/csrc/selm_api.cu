@@ -294,7 +294,7 @@ selm_status vcycle_t(selm_mg* h, Sys& s, int l, T* v0, const T* b0, bool noise, 
   // 527 per pass; 72^3: 831 and 757; 96^3: 1236 and 1076).  Those passes store the
   // same parity bits, so both forms give the same values.
   const bool flow_level = sizeof(T) == 4 && s.coop_flow && L.flow;
-  const bool full_passes = flow_level && L.c[0].ny > 1 && L.size > 1000000 && coarse_rows8(L);
+  const bool full_passes = flow_level && L.c[0].ny > 1 && L.size > 1000000 && coarse_row_pairs<T>(L);
   const bool coop = l > 0 && !last && !L.rb && level_sites(L) <= kCoopMaxSites && s.use_engine && s.use_coop &&
                     eng.valid && l < eng.params.l0 && s.coop_bar && level_coop_supported<T>(L);
   const bool tags = coop && full_passes;

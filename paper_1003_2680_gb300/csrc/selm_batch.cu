@@ -577,9 +577,13 @@ selm_status selm_batch_autotune(selm_batch* b, int* chosen_cluster, void* stream
     BCK(batch_persist_configure(b->bp, best_kc, best_bps));
     BST(check_timeout(b));
   }
-  // the per-system graph form over engine cluster sizes; the faster form wins
+  // the per-system graph form over engine cluster sizes; the faster form wins.
+  // A cluster too small for a level that the first candidate's engine holds is
+  // passed over: the level would run as per-pass launches, whose FP32 sums round
+  // differently, and the tuned batch would depend on the timing in its last bits.
   b->persistent = false;
   const int cands[3] = {16, 8, 4};
+  std::vector<int> first_level(b->n, -1);
   float best = -1.0f;
   int best_c = 0;
   cudaEvent_t e0, e1;
@@ -587,6 +591,14 @@ selm_status selm_batch_autotune(selm_batch* b, int* chosen_cluster, void* stream
   BCK(cudaEventCreate(&e1));
   for (int c : cands) {
     for (selm_mg* h : b->sys) BST(replan_engine(h, c, nullptr));
+    bool same_levels = true;
+    for (int i = 0; i < b->n; ++i) {
+      int l0 = 0;
+      selm_mg_engine_info(b->sys[i], SELM_SYS_VELOCITY, &l0, nullptr, nullptr);
+      if (c == cands[0]) first_level[i] = l0;
+      same_levels = same_levels && first_level[i] == l0;
+    }
+    if (!same_levels) continue;
     BST(build_cycle_graph(b));
     BCK(cudaGraphLaunch(b->g_cycle, st));   // warm-up
     BCK(cudaEventRecord(e0, st));

@@ -1211,7 +1211,7 @@ __global__ void __launch_bounds__(kBlock) k_coarse_site(LevelDev L, ColourPass c
 template <typename T, bool NOISE, int CX, bool CG>
 __device__ __forceinline__ void coarse_colour_v8_item(const LevelDev& L, const ColourPass& cp, const ColumnPass& sp,
                                                       T* __restrict__ v, const T* __restrict__ b, int sweep, Key key,
-                                                      unsigned long long cy, long long g, int tag = -1) {
+                                                      unsigned long long cy, long long g) {
   if (g >= sp.start[L.ncomp]) return;
   int ci = 0;
   while (ci + 1 < L.ncomp && g >= sp.start[ci + 1]) ++ci;
@@ -1288,19 +1288,155 @@ __device__ __forceinline__ void coarse_colour_v8_item(const LevelDev& L, const C
   for (int e = 0; e < 4; ++e) {
     T nv = ((CG ? __ldcg(b + rowi + 2 * e) : LdNC::ld(b + rowi + 2 * e)) - acc[e]) / diag;
     if (NOISE) nv += n4[e] / tsqrt(diag);
-    v[rowi + 2 * e] = tagged(nv, tag);
+    v[rowi + 2 * e] = nv;
   }
 }
 
 template <typename T, bool NOISE, int CX>
 __global__ void __launch_bounds__(kBlock) k_coarse_colour_v8(LevelDev L, ColourPass cp, ColumnPass sp,
                                                             T* __restrict__ v, const T* __restrict__ b, int sweep,
-                                                            Key key, const unsigned long long* __restrict__ cyc,
-                                                            int tag) {
+                                                            Key key, const unsigned long long* __restrict__ cyc) {
   pdl_enter();
   const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (g >= sp.start[L.ncomp]) return;
-  coarse_colour_v8_item<T, NOISE, CX, false>(L, cp, sp, v, b, sweep, key, NOISE ? *cyc : 0ull, g, tag);
+  coarse_colour_v8_item<T, NOISE, CX, false>(L, cp, sp, v, b, sweep, key, NOISE ? *cyc : 0ull, g);
+}
+
+// Both x colours of a class row in one launch (FP32, 8-wide rows of at most
+// 8 kBlock sites): the second colour couples to the first of the same launch
+// only through x +- 1 of its own row, so a block owns whole rows, keeps the first
+// colour's four updates of each 8-wide segment in registers and passes the one
+// at x0 + 8 through shared memory.  The row window is read once for both colours
+// and the segment written once.  Per site the arithmetic and order are
+// coarse_site_at's: of the second colour the z planes k + 1, k + 2 wait as (p1, p2)
+// until the own plane is known.  A pass is bound by the window's loads (15 rows of
+// 40 B per segment, from L2): both colours with their normals at 128^3 x 3 take 34 us
+// against 2 x 22 as two launches; the step at 192^3 (level 1 of 96^3) 12.3 ms against 13.4.
+struct RowPairs {
+  long long start[kMaxComps + 1];   // first class row of each component
+  int colour_id2[kMaxComps];        // the second colour's number (noise counter)
+};
+
+template <bool NOISE>
+__global__ void __launch_bounds__(kBlock, 2) k_coarse_rows8(LevelDev L, ColourPass cp, RowPairs rp,
+                                                           float* __restrict__ v, const float* __restrict__ b,
+                                                           int sweep, Key key,
+                                                           const unsigned long long* __restrict__ cyc, int tag) {
+  __shared__ float first[kBlock];
+  pdl_enter();
+  const int segs = L.c[0].nx >> 3, rpb = kBlock / segs;
+  const int r = threadIdx.x / segs, seg = threadIdx.x - r * segs;
+  const long long rows = rp.start[L.ncomp], row0 = (long long)blockIdx.x * rpb + r;
+  const bool act = r < rpb && row0 < rows;      // the others compute the last row and store nothing
+  const long long row = min(row0, rows - 1);
+  int ci = 0;
+  while (ci + 1 < L.ncomp && row >= rp.start[ci + 1]) ++ci;
+  const CompDev& c = L.c[ci];
+  const int nx = c.nx, ny = c.ny, nz = c.nz;
+  const unsigned lrow = (unsigned)(row - rp.start[ci]);
+  const int jj = (int)(lrow % (unsigned)cp.nyc[ci]), kk = (int)(lrow / (unsigned)cp.nyc[ci]);
+  const int j = cp.cy[ci] + c.my * jj, k = cp.cz[ci] + c.mz * kk;
+  const int x0 = seg << 3;
+  const int jm = j == 0 ? ny - 1 : j - 1, jp = j == ny - 1 ? 0 : j + 1;
+  const int xl = x0 == 0 ? nx - 1 : x0 - 1, xr = x0 + 8 == nx ? 0 : x0 + 8;
+  const float* zb = c.zb32 + k * 10;
+  const long long rowi = c.off + ((long long)k * ny + j) * nx + x0;
+  // r[1 + e] holds x0 + e
+  auto load = [&](int dz, float r0[10], float r1[10], float r2[10]) {
+    const float* vp = v + c.off + (long long)min(max(k + dz, 0), nz - 1) * ny * nx;
+    auto row10 = [&](const float* q, float w[10]) {
+      w[0] = q[xl];
+      Vec<float>::load8(q + x0, w + 1);
+      w[9] = q[xr];
+    };
+    row10(vp + (long long)j * nx, r1);
+    if (ny > 1) {
+      row10(vp + (long long)jm * nx, r0);
+      row10(vp + (long long)jp * nx, r2);
+    }
+  };
+  // the plane's two x-y sums at x0 + x
+  auto sums = [&](int x, bool centre, const float r0[10], const float r1[10], const float r2[10], float& p1, float& p2) {
+    if (ny == 1) {
+      p1 = c.w1f[3] * r1[x] + c.w1f[5] * r1[x + 2];
+      p2 = c.w2f[3] * r1[x] + c.w2f[5] * r1[x + 2];
+    } else {
+      p1 = c.w1f[0] * r0[x] + c.w1f[1] * r0[x + 1] + c.w1f[2] * r0[x + 2] + c.w1f[3] * r1[x] + c.w1f[5] * r1[x + 2] +
+           c.w1f[6] * r2[x] + c.w1f[7] * r2[x + 1] + c.w1f[8] * r2[x + 2];
+      p2 = c.w2f[0] * r0[x] + c.w2f[1] * r0[x + 1] + c.w2f[2] * r0[x + 2] + c.w2f[3] * r1[x] + c.w2f[5] * r1[x + 2] +
+           c.w2f[6] * r2[x] + c.w2f[7] * r2[x + 1] + c.w2f[8] * r2[x + 2];
+    }
+    if (centre) {
+      p1 += c.w1f[4] * r1[x + 1];
+      p2 += c.w2f[4] * r1[x + 1];
+    }
+  };
+  float acc[8], late1[2][4], late2[2][4], r0[10], r1[10], r2[10], own0[10], own[10], own2[10], p1, p2;
+#pragma unroll
+  for (int e = 0; e < 8; ++e) acc[e] = 0.f;
+#pragma unroll
+  for (int dz = -2; dz < 0; ++dz) {
+    load(dz, r0, r1, r2);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      sums(e, true, r0, r1, r2, p1, p2);
+      acc[e] += zb[dz + 2] * p1 + zb[5 + dz + 2] * p2;
+    }
+  }
+  load(0, own0, own, own2);
+#pragma unroll
+  for (int e = 0; e < 8; e += 2) {
+    sums(e, false, own0, own, own2, p1, p2);
+    acc[e] += zb[2] * p1 + zb[7] * p2;
+  }
+#pragma unroll
+  for (int dz = 1; dz <= 2; ++dz) {
+    load(dz, r0, r1, r2);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      sums(e, true, r0, r1, r2, p1, p2);
+      if (e & 1) {
+        late1[dz - 1][e >> 1] = p1;
+        late2[dz - 1][e >> 1] = p2;
+      } else {
+        acc[e] += zb[dz + 2] * p1 + zb[5 + dz + 2] * p2;
+      }
+    }
+  }
+  float bb[8], n4[2][4];
+  Vec<float>::load8(b + rowi, bb);
+  const float diag = coarse_diag<float>(c, k);
+  if (NOISE) {
+    const unsigned long long cy = *cyc;
+    const unsigned grp = (unsigned)seg + (unsigned)(cp.nxc[ci] >> 2) * (unsigned)(jj + cp.nyc[ci] * kk);
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      Normals<float>::get(philox10(make_uint4(grp, ctr1_of(L.level, c.comp_id, h ? rp.colour_id2[ci] : cp.colour_id[ci],
+                                                           sweep, 0),
+                                              (uint32_t)cy, (uint32_t)(cy >> 32)),
+                                   key.k0, key.k1),
+                          n4[h]);
+  }
+  auto update = [&](int e) {
+    float nv = (bb[e] - acc[e]) / diag;
+    if (NOISE) nv += n4[e & 1][e >> 1] / tsqrt(diag);
+    return tagged(nv, tag);
+  };
+#pragma unroll
+  for (int e = 0; e < 8; e += 2) own[1 + e] = update(e);
+  first[threadIdx.x] = own[1];
+  __syncthreads();
+  if (act) own[9] = first[seg + 1 == segs ? threadIdx.x - seg : threadIdx.x + 1];
+#pragma unroll
+  for (int e = 1; e < 8; e += 2) {
+    sums(e, false, own0, own, own2, p1, p2);
+    acc[e] += zb[2] * p1 + zb[7] * p2;
+    acc[e] += zb[3] * late1[0][e >> 1] + zb[8] * late2[0][e >> 1];
+    acc[e] += zb[4] * late1[1][e >> 1] + zb[9] * late2[1][e >> 1];
+  }
+#pragma unroll
+  for (int e = 1; e < 8; e += 2) own[1 + e] = update(e);
+  if (act) Vec<float>::store8(v + rowi, own + 1);
 }
 
 // ---------------------------------------------------------------------------
@@ -3091,6 +3227,20 @@ bool coarse_rows8(const LevelDev& L) {
   return true;
 }
 
+// Such rows, of one length and within a block, in FP32: two colours per launch
+// (k_coarse_rows8).  FP64 keeps a launch per colour: its narrow pipe bounds the
+// pass, which the window read once does not relieve.  The x colour is the
+// fastest digit of a colour's number, so colours q, q + 1 (q even) share their rows.
+template <typename T>
+bool coarse_row_pairs(const LevelDev& L) {
+  if (sizeof(T) != 4 || !coarse_rows8(L) || L.c[0].nx > 8 * kBlock) return false;
+  for (int ci = 0; ci < L.ncomp; ++ci)
+    if (L.c[ci].nx != L.c[0].nx || L.c[ci].ncol % 2 != 0) return false;
+  return true;
+}
+template bool coarse_row_pairs<float>(const LevelDev&);
+template bool coarse_row_pairs<double>(const LevelDev&);
+
 template <typename T>
 cudaError_t launch_smooth(const LevelDev& L, T* v, const T* b, int sweep, bool noise, Key key,
                           const unsigned long long* cyc, cudaStream_t st, int tag) {
@@ -3158,13 +3308,34 @@ cudaError_t launch_smooth(const LevelDev& L, T* v, const T* b, int sweep, bool n
   int maxcol = 0;
   for (int ci = 0; ci < L.ncomp; ++ci) maxcol = maxcol > L.c[ci].ncol ? maxcol : L.c[ci].ncol;
   const bool v8 = coarse_rows8(L);
-  if (tag >= 0 && !v8) return cudaErrorNotSupported;
+  if (tag >= 0 && !coarse_row_pairs<T>(L)) return cudaErrorNotSupported;
   for (int q = 0; q < maxcol; ++q) {
     ColourPass cp{};
     const long long gs = colour_pass_of(L, q, &cp);
     if (gs == 0) continue;
     prof::Scope ps(SELM_K_COARSE_SWEEP, st);
-    if (v8) {
+    if constexpr (std::is_same<T, float>::value) {
+      if (coarse_row_pairs<T>(L)) {   // colours q (x even) and q + 1 (x odd)
+        ColourPass cp2{};
+        colour_pass_of(L, q + 1, &cp2);
+        RowPairs rp{};
+        long long rows = 0;
+        for (int ci = 0; ci < L.ncomp; ++ci) {
+          rp.start[ci] = rows;
+          if (cp.nsites[ci] > 0) rows += (long long)cp.nyc[ci] * cp.nzc[ci];
+          rp.colour_id2[ci] = cp2.colour_id[ci];
+        }
+        rp.start[L.ncomp] = rows;
+        const int rpb = kBlock / (L.c[0].nx >> 3);
+        const unsigned grid = (unsigned)((rows + rpb - 1) / rpb);
+        if (noise)
+          LTRY(launch_pdl(k_coarse_rows8<true>, grid, kBlock, st, L, cp, rp, v, b, sweep, key, cyc, tag));
+        else
+          LTRY(launch_pdl(k_coarse_rows8<false>, grid, kBlock, st, L, cp, rp, v, b, sweep, key, cyc, tag));
+        ++q;
+        continue;
+      }
+    } else if (v8) {
       ColumnPass sp{};
       long long items = 0;
       for (int ci = 0; ci < L.ncomp; ++ci) {
@@ -3174,17 +3345,13 @@ cudaError_t launch_smooth(const LevelDev& L, T* v, const T* b, int sweep, bool n
       sp.start[L.ncomp] = items;
       const int cx = q % 2;   // every component has x modulus 2
       if (noise && cx == 0)
-        LTRY(launch_pdl(k_coarse_colour_v8<T, true, 0>, grid_for(items), kBlock, st, L, cp, sp, v, b, sweep, key, cyc,
-                        tag));
+        LTRY(launch_pdl(k_coarse_colour_v8<T, true, 0>, grid_for(items), kBlock, st, L, cp, sp, v, b, sweep, key, cyc));
       else if (noise)
-        LTRY(launch_pdl(k_coarse_colour_v8<T, true, 1>, grid_for(items), kBlock, st, L, cp, sp, v, b, sweep, key, cyc,
-                        tag));
+        LTRY(launch_pdl(k_coarse_colour_v8<T, true, 1>, grid_for(items), kBlock, st, L, cp, sp, v, b, sweep, key, cyc));
       else if (cx == 0)
-        LTRY(launch_pdl(k_coarse_colour_v8<T, false, 0>, grid_for(items), kBlock, st, L, cp, sp, v, b, sweep, key, cyc,
-                        tag));
+        LTRY(launch_pdl(k_coarse_colour_v8<T, false, 0>, grid_for(items), kBlock, st, L, cp, sp, v, b, sweep, key, cyc));
       else
-        LTRY(launch_pdl(k_coarse_colour_v8<T, false, 1>, grid_for(items), kBlock, st, L, cp, sp, v, b, sweep, key, cyc,
-                        tag));
+        LTRY(launch_pdl(k_coarse_colour_v8<T, false, 1>, grid_for(items), kBlock, st, L, cp, sp, v, b, sweep, key, cyc));
       continue;
     }
     if (noise)

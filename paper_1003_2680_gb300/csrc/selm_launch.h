@@ -51,7 +51,8 @@ inline int z_chunk(long long cols, int nz, int esize) {
 // launch_smooth's tag (Galerkin levels with coarse_rows8()): 0 or 1, the parity
 // bit that FP32 updates store in dataflow order (launch_level_coop); -1: none.
 // launch_prolong's tag0 clears the bit (update count 0).
-bool coarse_rows8(const LevelDev& L);
+template <typename T>
+bool coarse_row_pairs(const LevelDev& L);
 template <typename T>
 cudaError_t launch_smooth(const LevelDev& L, T* v, const T* b, int sweep, bool noise, Key key,
                           const unsigned long long* cyc, cudaStream_t st, int tag = -1);

@@ -54,3 +54,22 @@ def test_full_passes_keep_dataflow_values(noise):
         out.append(v)
     assert ((out[0] - out[1]).norm() / out[1].norm()).item() < 1e-5
     assert not torch.equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("dim,n", [(3, 48), (3, 80), (2, 208), (2, 1024)])
+@pytest.mark.parametrize("noise", [0, 1])
+def test_row_pairs(dim, n, noise):
+    """Both x colours of a row in one launch: rows of 3, 5, 13 and 64 segments (a
+    block's last threads idle, the neighbour segment wraps), one sweep of level 1."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from oracle import gibbs
+    from paper_1003_2680_gb300 import selm as S
+    m = S.SelmMG(dim=dim, n=n, levels=2, precision=1, coarse_mode=1, seed=11, instance=3)
+    osys = grid.velocity_system(n, dim, levels=2)
+    v0 = round_like(selm_inputs.fields(osys.shapes(1), seed=1), torch.float32)
+    b0 = round_like(selm_inputs.fields(osys.shapes(1), seed=2), torch.float32)
+    v, b = to_dev(m.h, v0, torch.float32, level=1), to_dev(m.h, b0, torch.float32, level=1)
+    S.selm_mg_smooth(m.h, 0, 1, v, b, sweep=1, cycle=7, noise=noise)
+    want = gibbs.sweep(osys, 1, [x.copy() for x in v0], b0, 1, philox.PhiloxNoise(11, 3, 7), float(noise))
+    assert rel(from_dev(m.h, v, level=1), want) < 1e-5
