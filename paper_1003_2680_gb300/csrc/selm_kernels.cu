@@ -248,6 +248,21 @@ __device__ __forceinline__ double block_sum(double x) {
   return x;
 }
 
+// The same over B threads with the first warp alone adding: B / 32 - 1 + 5 FP64
+// adds a block instead of five in each warp, for kernels that the FP64 pipe bounds.
+template <int B>
+__device__ __forceinline__ double block_sum_first(double x) {
+  __shared__ double red[B];
+  red[threadIdx.x] = x;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+#pragma unroll
+    for (int q = 32; q < B; q += 32) x += red[threadIdx.x + q];
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+  }
+  return x;
+}
+
 // Level 0, red-black, vectorised: one thread owns the 8 consecutive x
 // positions [8g, 8g+8) of one row (requires nx % 8 == 0).  These hold exactly
 // the four sites of colour `colour` of one noise group (ranks 4g'..4g'+3 of
@@ -361,43 +376,56 @@ __device__ __forceinline__ long long fx_align(long long bits, int emax) {
   return d >= 63 ? (m < 0 ? -1ll : 0ll) : ((m * 32) >> d);
 }
 
+// The same for a window of exponents within 31 of emax (none zero), one 64-bit
+// shift by less than 32, the magnitude truncated; the caller adds neg.
+__device__ __forceinline__ unsigned long long fx_align31(long long bits, unsigned emax20, unsigned* neg) {
+  const unsigned hi = (unsigned)((unsigned long long)bits >> 32), lo = (unsigned)bits;
+  const unsigned sh = (emax20 - (hi & 0x7ff00000u)) >> 20;
+  const unsigned mh = (hi & 0x000fffffu) | 0x00100000u;
+  const unsigned h5 = __funnelshift_l(lo, mh, 5), l5 = lo << 5;
+  const unsigned s = (unsigned)((int)hi >> 31);   // all ones for a negative value
+  *neg = s;
+  return ((unsigned long long)((h5 >> sh) ^ s) << 32) | (__funnelshift_r(l5, h5, sh) ^ s);
+}
+
 // S 2^e2 rounded to nearest even as FP64 (S != 0 and the result normal,
-// which the caller's exponent guard ensures).
+// which the caller's exponent guard ensures).  The leading one of the shifted
+// magnitude and a carry out of the rounding both add into the exponent field.
 __device__ __forceinline__ double fx_to_double(long long S, int e2) {
-  const unsigned long long sign = S < 0 ? 0x8000000000000000ull : 0ull;
-  unsigned long long a = S < 0 ? (unsigned long long)(-S) : (unsigned long long)S;
+  const long long sgn = S >> 63;
+  unsigned long long a = (unsigned long long)((S ^ sgn) - sgn);
   const int lz = __clzll((long long)a);
   a <<= lz;
-  unsigned long long mant = a >> 11;
-  const unsigned long long rem = a & 0x7ffull;
-  int E = 63 - lz + e2;
-  if (rem > 0x400ull || (rem == 0x400ull && (mant & 1ull))) {
-    ++mant;
-    if (mant >> 53) {
-      mant >>= 1;
-      ++E;
-    }
-  }
-  return __longlong_as_double((long long)(sign | ((unsigned long long)(E + 1023) << 52) | (mant & 0x000FFFFFFFFFFFFFull)));
+  const unsigned lo = (unsigned)a;
+  const unsigned up = (lo & 0x7ffu) + ((lo >> 11) & 1u) > 0x400u ? 1u : 0u;
+  const unsigned long long mag = (a >> 11) + up + ((unsigned long long)(unsigned)(63 - lz + e2 + 1022) << 52);
+  return __longlong_as_double((long long)(mag | ((unsigned long long)sgn & 0x8000000000000000ull)));
 }
 
 // FP64 -> FP32, round to nearest even, by integer operations on the normal
-// FP32 range; other values through the conversion instruction.
+// FP32 range; other values through the conversion instruction.  Written out as
+// assembly it stays in its branch: the compiler otherwise issues it for every
+// value and selects.
 __device__ __forceinline__ float fx_to_float(double x) {
-  const long long b = __double_as_longlong(x);
-  const int ex = fx_exp(b);
-  if (ex < 1023 - 126 || ex > 1023 + 127) return __double2float_rn(x);
-  const unsigned long long mant = (unsigned long long)b & 0x000FFFFFFFFFFFFFull;
-  const unsigned m23 = (unsigned)(mant >> 29);
-  const unsigned long long rem = mant & 0x1FFFFFFFull;
-  unsigned f = ((unsigned)((unsigned long long)b >> 32) & 0x80000000u) | ((unsigned)(ex - 1023 + 127) << 23) | m23;
-  if (rem > 0x10000000ull || (rem == 0x10000000ull && (m23 & 1u))) f += 1u;
-  return __uint_as_float(f);
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned ex = (hi >> 20) & 0x7ffu;
+  if (ex - 897u > 253u) {
+    float f;
+    asm volatile("cvt.rn.f32.f64 %0, %1;" : "=f"(f) : "d"(x));
+    return f;
+  }
+  const unsigned m = ((ex - 896u) << 23) | __funnelshift_l(lo, hi & 0xfffffu, 3);
+  const unsigned rem = lo << 3;   // the dropped 29 bits from the top
+  return __uint_as_float((hi & 0x80000000u) | (m + (rem > 0x80000000u - (m & 1u) ? 1u : 0u)));
 }
 
-// The FP32-output residual of k_outer_residual_v4 in the exact form above.
+// The FP32-output residual of k_outer_residual_v4 in the exact form above.  128^3
+// (3 components, with the norm): 69 us, bound by the integer pipe at 150
+// instructions per unknown; 84 us with 180 of them and the norm summed by FP64
+// shuffles in every warp of 256-thread blocks (a third of the FP64 work).
+constexpr int kFxBlock = 128;
 template <bool NORM>
-__global__ void __launch_bounds__(kBlock) k_outer_residual_fx(LevelDev L, RowPass rp, const double* __restrict__ z,
+__global__ void __launch_bounds__(kFxBlock, 5) k_outer_residual_fx(LevelDev L, RowPass rp, const double* __restrict__ z,
                                                              const double* __restrict__ b, float* __restrict__ r,
                                                              double* __restrict__ norm2) {
   pdl_enter();
@@ -417,8 +445,8 @@ __global__ void __launch_bounds__(kBlock) k_outer_residual_fx(LevelDev L, RowPas
     const long long rbase = c.off + (long long)row * nx;
     const int x0 = seg << 2;
     // the window as FP64 bit patterns: the centre row (4, left, right), then
-    // the rows y-1, y+1, z-1, z+1 in fixed slots, an absent row as zeros
-    // (which add nothing and do not raise the window's exponent)
+    // the rows y-1, y+1, z-1, z+1 in fixed slots; an absent row repeats the centre
+    // row, which leaves the window's exponents alone, and is not summed
     long long w[22];
     auto ld4 = [&](bool present, long long off, long long* dst) {
       if (present) {
@@ -426,7 +454,7 @@ __global__ void __launch_bounds__(kBlock) k_outer_residual_fx(LevelDev L, RowPas
         const longlong2 d = *reinterpret_cast<const longlong2*>(z + off + 2);
         dst[0] = a.x; dst[1] = a.y; dst[2] = d.x; dst[3] = d.y;
       } else {
-        dst[0] = 0; dst[1] = 0; dst[2] = 0; dst[3] = 0;
+        dst[0] = w[0]; dst[1] = w[1]; dst[2] = w[2]; dst[3] = w[3];
       }
     };
     ld4(true, rbase + x0, w);
@@ -437,14 +465,20 @@ __global__ void __launch_bounds__(kBlock) k_outer_residual_fx(LevelDev L, RowPas
     ld4(ys, c.off + ((long long)k * c.ny + (j == c.ny - 1 ? 0 : j + 1)) * nx + x0, w + 10);
     ld4(k > 0, rbase - plane + x0, w + 14);
     ld4(k < c.nz - 1, rbase + plane + x0, w + 18);
-    int emax = 0;
+    const bool present[4] = {ys, ys, k > 0, k < c.nz - 1};
+    unsigned emax20 = 0u, emin20 = 0x7ff00000u;   // exponents where they stand in the high word
 #pragma unroll
-    for (int q = 0; q < 22; ++q) emax = max(emax, fx_exp(w[q]));
+    for (int q = 0; q < 22; ++q) {
+      const unsigned e20 = (unsigned)((unsigned long long)w[q] >> 32) & 0x7ff00000u;
+      emax20 = max(emax20, e20);
+      emin20 = min(emin20, e20);
+    }
+    const int emax = (int)(emax20 >> 20);
     const int edges = (k == 0) + (k == c.nz - 1);
     int dz = 2;
     if (c.zkind == kAxisCellDir) dz += edges;
     if (c.zkind == kAxisCellNeu) dz -= edges;
-    const long long dg = (c.ny > 1 ? 4 : 2) + dz;
+    const int dg = (c.ny > 1 ? 4 : 2) + dz;
     double bv[4] = {0.0, 0.0, 0.0, 0.0};
     if (b) {
       const double2 a = *reinterpret_cast<const double2*>(b + rbase + x0);
@@ -457,21 +491,40 @@ __global__ void __launch_bounds__(kBlock) k_outer_residual_fx(LevelDev L, RowPas
 #pragma unroll
       for (int e = 0; e < 4; ++e) res[e] = bv[e];
     } else if (emax >= 64 && emax <= 2000) {
-      long long Z[22];
+      // S = the neighbours' sum, C = the centre
+      unsigned long long S[4], C[4];
+      if (emin20 != 0u && emax20 - emin20 <= (31u << 20)) {
+        unsigned n[22];
+        unsigned long long Z[22];
 #pragma unroll
-      for (int q = 0; q < 22; ++q) Z[q] = fx_align(w[q], emax);
-      long long S[4];
-      S[0] = Z[4] + Z[1];
-      S[1] = Z[0] + Z[2];
-      S[2] = Z[1] + Z[3];
-      S[3] = Z[2] + Z[5];
+        for (int q = 0; q < 22; ++q) Z[q] = fx_align31(w[q], emax20, &n[q]);
 #pragma unroll
-      for (int q = 6; q < 22; q += 4) {
-        S[0] += Z[q]; S[1] += Z[q + 1]; S[2] += Z[q + 2]; S[3] += Z[q + 3];
+        for (int e = 0; e < 4; ++e) {
+          C[e] = Z[e] - (long long)(int)n[e];
+          const int l = e == 0 ? 4 : e - 1, r = e == 3 ? 5 : e + 1;
+          S[e] = Z[l] + Z[r];
+          int neg = (int)n[l] + (int)n[r];
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (present[q]) {
+              S[e] += Z[6 + 4 * q + e];
+              neg += (int)n[6 + 4 * q + e];
+            }
+          S[e] -= (long long)neg;
+        }
+      } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          C[e] = (unsigned long long)fx_align(w[e], emax);
+          S[e] = (unsigned long long)(fx_align(w[e == 0 ? 4 : e - 1], emax) + fx_align(w[e == 3 ? 5 : e + 1], emax));
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (present[q]) S[e] += (unsigned long long)fx_align(w[6 + 4 * q + e], emax);
+        }
       }
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        const long long t = dg * Z[e] - S[e];
+        const long long t = (long long)((unsigned long long)dg * C[e] - S[e]);
         const double az = t == 0 ? 0.0 : fx_to_double(t, emax - 1080);
         res[e] = fma(-c.s, az, bv[e]);
       }
@@ -485,9 +538,9 @@ __global__ void __launch_bounds__(kBlock) k_outer_residual_fx(LevelDev L, RowPas
       acc[2] = cz[1] + cz[3];
       acc[3] = cz[2] + cz[5];
 #pragma unroll
-      for (int q = 6; q < 22; q += 4) {
-        acc[0] += cz[q]; acc[1] += cz[q + 1]; acc[2] += cz[q + 2]; acc[3] += cz[q + 3];
-      }
+      for (int q = 0; q < 4; ++q)
+        if (present[q])
+          for (int e = 0; e < 4; ++e) acc[e] += cz[6 + 4 * q + e];
       const double sdg = c.s * (double)dg;
 #pragma unroll
       for (int e = 0; e < 4; ++e) res[e] = fma(c.s, acc[e], fma(-sdg, cz[e], bv[e]));
@@ -500,7 +553,7 @@ __global__ void __launch_bounds__(kBlock) k_outer_residual_fx(LevelDev L, RowPas
     *reinterpret_cast<float4*>(r + rbase + x0) = make_float4(out[0], out[1], out[2], out[3]);
   }
   if (NORM) {
-    rr = block_sum(rr);
+    rr = block_sum_first<kFxBlock>(rr);
     if (threadIdx.x == 0) atomicAdd(norm2, rr);
   }
 }
@@ -3575,9 +3628,9 @@ cudaError_t launch_outer_residual(const LevelDev& L0, const double* z, const dou
       else if (!aligned)
         LTRY(launch_pdl(k_outer_residual_v4<T, false>, grid_for(nt), kBlock, st, L0, rp, z, b, r, norm2));
       else if (norm2)
-        LTRY(launch_pdl(k_outer_residual_fx<true>, grid_for(nt), kBlock, st, L0, rp, z, b, r, norm2));
+        LTRY(launch_pdl(k_outer_residual_fx<true>, grid_for(nt, kFxBlock), kFxBlock, st, L0, rp, z, b, r, norm2));
       else
-        LTRY(launch_pdl(k_outer_residual_fx<false>, grid_for(nt), kBlock, st, L0, rp, z, b, r, norm2));
+        LTRY(launch_pdl(k_outer_residual_fx<false>, grid_for(nt, kFxBlock), kFxBlock, st, L0, rp, z, b, r, norm2));
       return cudaGetLastError();
     }
     if (norm2)

@@ -65,8 +65,8 @@ def test_row_pairs(dim, n, noise):
         pytest.skip("no CUDA device")
     from oracle import gibbs
     from paper_1003_2680_gb300 import selm as S
-    m = S.SelmMG(dim=dim, n=n, levels=2, precision=1, coarse_mode=1, seed=11, instance=3)
-    osys = grid.velocity_system(n, dim, levels=2)
+    m = S.SelmMG(dim=dim, n=n, precision=1, seed=11, instance=3)
+    osys = grid.velocity_system(n, dim, levels=S.selm_mg_levels(m.h))
     v0 = round_like(selm_inputs.fields(osys.shapes(1), seed=1), torch.float32)
     b0 = round_like(selm_inputs.fields(osys.shapes(1), seed=2), torch.float32)
     v, b = to_dev(m.h, v0, torch.float32, level=1), to_dev(m.h, b0, torch.float32, level=1)
