@@ -286,18 +286,22 @@ selm_status vcycle_t(selm_mg* h, Sys& s, int l, T* v0, const T* b0, bool noise, 
   const EnginePlanT<T>& eng = eng_of<T>(s);
   // A level above the engine with at most 2^20 sites per component: each half
   // of its V-cycle in one cooperative launch (one or a few site updates per
-  // thread per pass).  Larger levels keep one GPU-wide launch per colour pass,
-  // whose parallelism then beats the launch overhead.  In dataflow order that
-  // already holds for 3-D levels of more than a million unknowns: a pass costs
-  // about 3 us of update latency plus its sites over 78 K threads, a launch per
-  // pass less once it is full (V-cycle with level 1 of 64^3 446 us cooperative,
-  // 527 per pass; 72^3: 831 and 757; 96^3: 1236 and 1076).  Those passes store the
-  // same parity bits, so both forms give the same values.
+  // thread per pass).  Larger levels keep GPU-wide launches per pass, whose
+  // parallelism then beats the launch overhead.  Where a launch updates both x
+  // colours of a row that already holds
+  //  - in 2-D, three such launches a sweep against six grid barriers (V-cycle with
+  //    level 1 of 384^2 256 us cooperative, 227 with launches; 512^2: 326 and 267;
+  //    768^2: 517 and 403; two levels, of 1024^2 and 512^2: 756 and 522);
+  //  - in 3-D for levels of more than a million unknowns: in dataflow order a pass
+  //    costs about 3 us of update latency plus its sites over 78 K threads (64^3: 446
+  //    cooperative, 473 with launches; 72^3: 854 and 684; 80^3: 849 and 743).
+  // Launches for a level in dataflow order store the same parity bits, so both
+  // forms give the same values.
   const bool flow_level = sizeof(T) == 4 && s.coop_flow && L.flow;
-  const bool full_passes = flow_level && L.c[0].ny > 1 && L.size > 1000000 && coarse_row_pairs<T>(L);
+  const bool full_passes = coarse_row_pairs<T>(L) && (L.c[0].ny == 1 || (flow_level && L.size > 1000000));
   const bool coop = l > 0 && !last && !L.rb && level_sites(L) <= kCoopMaxSites && s.use_engine && s.use_coop &&
                     eng.valid && l < eng.params.l0 && s.coop_bar && level_coop_supported<T>(L);
-  const bool tags = coop && full_passes;
+  const bool tags = coop && full_passes && flow_level;
   if (coop && !full_passes) {
     const LevelDev& Lc = s.lev[l + 1];
     CK(launch_level_coop<T>(L, Lc, 0, h->mu1, h->mu2, v, b, (T*)s.t[l], (T*)s.b[l + 1], (T*)s.v[l + 1], s.coop_bar,

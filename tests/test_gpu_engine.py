@@ -73,3 +73,23 @@ def test_row_pairs(dim, n, noise):
     S.selm_mg_smooth(m.h, 0, 1, v, b, sweep=1, cycle=7, noise=noise)
     want = gibbs.sweep(osys, 1, [x.copy() for x in v0], b0, 1, philox.PhiloxNoise(11, 3, 7), float(noise))
     assert rel(from_dev(m.h, v, level=1), want) < 1e-5
+
+
+@pytest.mark.parametrize("n", [768, 2048])
+def test_2d_levels_by_launches(n):
+    """2-D levels above the engine: launches of row pairs by default; the cooperative
+    option set explicitly or off makes no difference to any value."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1003_2680_gb300 import selm as S
+    m = S.SelmMG(dim=2, n=n, precision=1, seed=11, instance=3)
+    assert S.selm_mg_engine_info(m.h)[0] >= 2
+    b = torch.randn(comps(m.h, 0, 0)[1], device="cuda", generator=torch.Generator("cuda").manual_seed(5))
+    out = []
+    for coop in (1, 0):
+        S.selm_mg_set_option(m.h, S.SELM_OPT_LEVEL_COOP, coop)
+        S.selm_mg_set_option(m.h, S.SELM_OPT_ENGINE_LEVEL, 2)
+        v = torch.zeros_like(b)
+        S.selm_mg_vcycle(m.h, 0, v, b, 7, 1)
+        out.append(v)
+    assert ((out[0] - out[1]).norm() / out[1].norm()).item() < 1e-5
