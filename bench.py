@@ -1082,7 +1082,8 @@ def stokes_measure(S, n, particles, steps, warmup):
     each step = the random-finite-difference drift (two Stokes mobility
     solves), 2 chain cycles and one Stokes solve of the combined forced and
     thermal field.  Every Stokes solve is conjugate gradients on the pressure
-    Schur complement with FAC inner solves."""
+    Schur complement; its inner solves are FP64 refinement around the spectral
+    solve (power-of-two channels), else FAC cycles."""
     import torch
     import selm_inputs
     d = S.make_desc(dim=3, n=n, kT=1.0, precision=S.SELM_FP32_REFINE64, seed=0, instance=0,

@@ -173,14 +173,16 @@ enum {
    first level whose slabs fit in shared memory); the levels above it run as
    GPU-wide launches.  Re-plans both systems' engines.
    SELM_OPT_LEVEL_COOP (default 1): each half V-cycle of a level above the
-   engine runs as one cooperative launch over every SM.  1: with FP32 inner
+   engine runs as one cooperative launch over every SM (FP32 levels in 2-D, and
+   of more than a million unknowns in 3-D, as launches of two colours each, with
+   the cooperative form's values).  1: with FP32 inner
    cycles the colour passes run in dataflow order, each site update waiting
    for its coupled neighbours only (each stored value carries the parity of
    its update count in its least significant mantissa bit, at most 1 ulp from
    the rounded update); FP64 levels, and levels whose stencil admits no such
    order, separate the passes by grid barriers.  2: grid barriers always.
    Every wait is bounded; a timed-out wait is reported as SELM_ECUDA by the
-   next solve's norm read.  0 selects one launch per colour pass.  All give
+   next solve's norm read.  0 selects launches per colour pass.  All give
    the same result up to rounding. */
 /* SELM_OPT_GRAPHS (default 1): the V-cycles of solves and chain cycles on the
    handle's own buffers are captured once as CUDA graphs (on a stream of the
@@ -426,8 +428,10 @@ selm_status selm_server_destroy(selm_server* s);
    M = Gamma P~ A^-1 P~ Gamma^T and drops kT div_X M, Section 2.1).
    selm_mg_stokes_solve: u = S f, the velocity of the MAC saddle point
    A u + D^T p = f, D u = 0 (D the integer MAC divergence), by conjugate
-   gradients on the pressure Schur complement D A^-1 D^T with FAC inner solves
-   (Algorithm 1) a hundred times tighter than `tol` (0: the descriptor's tol);
+   gradients on the pressure Schur complement D A^-1 D^T with inner solves a
+   hundred times tighter than `tol` (0: the descriptor's tol): FP64 refinement
+   around the channel operator's spectral solve where the grid has one, else FAC
+   cycles (Algorithm 1);
    f, u: device velocity fields (level-0 layout).  iters / resid (optional
    HOST) receive the outer iterations and the relative Schur residual; the
    call synchronises.  The first Stokes call allocates the handle's Stokes
