@@ -3400,7 +3400,8 @@ cudaError_t launch_smooth(const LevelDev& L, T* v, const T* b, int sweep, bool n
         ++q;
         continue;
       }
-    } else if (v8) {
+    }
+    if (v8) {   // FP64, and FP32 rows wider than a block
       ColumnPass sp{};
       long long items = 0;
       for (int ci = 0; ci < L.ncomp; ++ci) {

@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(kThreads) k_colour(SellDev S, int pos0, int cn
     rd = rd_at<T>(S, p);
     if (NK != 0) {
       T gn;
-      if (drawn) {
+      if (sizeof(T) == 8 && drawn) {   // (FP32 cycles draw at the rows)
         gn = drawn[p];
       } else {
         const unsigned long long c = *cyc;
@@ -389,7 +389,7 @@ __device__ __forceinline__ void row_lane_load(const SellDev& S, int g, int pos0,
       k.rd = rd_at<T>(S, p);
       if (NK != 0) {
         T gn;
-        if (drawn) {
+        if (sizeof(T) == 8 && drawn) {   // (FP32 cycles draw at the rows)
           gn = drawn[p];
         } else {
           const uint4 wv = philox4x32_10(make_uint4((uint32_t)t >> 2, c1, (uint32_t)c64, (uint32_t)(c64 >> 32)),
@@ -580,7 +580,8 @@ __global__ void __launch_bounds__(kThreads) k_scale(long long n, const double* _
   if (i < n) y[i] = DIV ? x[i] / s[i] : x[i] * s[i];
 }
 
-// Conjugate gradients (Jacobi preconditioned) on diag(vol) L phi = rhs, the
+// Preconditioned conjugate gradients (by the diagonal, or by the spectral solve
+// further down) on diag(vol) L phi = rhs, the
 // scalars kept on the device: sc[0], sc[1] = r.z of even / odd iterations,
 // sc[2] = the starting r.z, sc[3] = r.r.  An iteration is three launches
 // (programmatic dependent launches): q = S p with the partial sums of p.q;
