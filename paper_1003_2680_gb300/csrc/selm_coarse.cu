@@ -781,8 +781,9 @@ __device__ void stage_colours(const EngLevel<T>& L, int z0, int z1, EngColour* c
 // The normals of every sweep of the levels that the plan gave a buffer, drawn
 // once at the start of the launch by all threads, a whole Philox block at a
 // time: a cluster level's by the CTA that owns the planes, CTA 0's levels by
-// all CTAs of the cluster (through distributed shared memory).  The cluster
-// barrier before the first use orders them.  Normal of (sweep, class, rank)
+// all CTAs of the cluster (through distributed shared memory; called behind a
+// cluster barrier, since a CTA's shared memory may be written only once it
+// runs).  The cluster barrier before the first use orders them.  Normal of (sweep, class, rank)
 // at [sweep * sites per CTA + the class's offset + rank - its first rank].
 template <typename T>
 __device__ void stage_noise(const EngParams<T>* P, const EngRun& run, unsigned char* smem, const EngLevel<T>* lev0,
@@ -844,6 +845,9 @@ __global__ void __launch_bounds__(EngThreads<T>::value, 1) k_coarse_engine(const
   cg::cluster_group cl = cg::this_cluster();
   const int csize = (int)cl.num_blocks();
   const int rank = (int)cl.block_rank();
+  // stage_noise() stores into CTA 0's shared memory: every CTA of the cluster
+  // has to run before the first store (the wait stands in front of it)
+  if (NOISE && csize > 1) cl.barrier_arrive();
   const int comp = blockIdx.x / csize;
   const EngComp<T>* E = &P->comp[comp];
   const unsigned long long cyc = *run.cyc;
@@ -960,7 +964,10 @@ __global__ void __launch_bounds__(EngThreads<T>::value, 1) k_coarse_engine(const
     w.col = col_at(l);
     return w;
   };
-  if (NOISE) stage_noise<T>(P, run, smem, lev0, col0, rank, csize, cyc);
+  if (NOISE) {
+    if (csize > 1) cl.barrier_wait();
+    stage_noise<T>(P, run, smem, lev0, col0, rank, csize, cyc);
+  }
   // the sweeps of level l from sweep index `first`, with b in shared memory
   // (blocal) or read from L2
   auto pass_args = [&](int l, int first, const T* b, bool blocal, int boff) {

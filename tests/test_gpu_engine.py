@@ -93,3 +93,30 @@ def test_2d_levels_by_launches(n):
         S.selm_mg_vcycle(m.h, 0, v, b, 7, 1)
         out.append(v)
     assert ((out[0] - out[1]).norm() / out[1].norm()).item() < 1e-5
+
+
+@pytest.mark.parametrize("dim,n,prec", [(2, 32, "fp64"), (2, 32, "fp32"), (2, 64, "fp64"), (3, 48, "fp32")])
+def test_normals_drawn_into_another_block(dim, n, prec):
+    """The engine's normals reach the block that holds a level from the other blocks
+    of its cluster: with no level divided over the cluster (2-D, 16^2 and below: the
+    others are there to draw only) and beside levels that are.  Many launches one
+    after another, each with its own counter, against the oracle."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1003_2680_gb300 import selm as S
+    dt, tol = (torch.float64, 1e-12) if prec == "fp64" else (torch.float32, 1e-5)
+    m = S.SelmMG(dim=dim, n=n, precision=0 if prec == "fp64" else 1, seed=11, instance=3)
+    assert S.selm_mg_engine_info(m.h)[0] == 1
+    osys = grid.velocity_system(n, dim, levels=S.selm_mg_levels(m.h))
+    v0 = round_like(selm_inputs.fields(osys.shapes(0), seed=1), dt)
+    b0 = round_like(selm_inputs.fields(osys.shapes(0), seed=2), dt)
+    b = to_dev(m.h, b0, dt)
+    out = []
+    for cycle in range(64):
+        v = to_dev(m.h, v0, dt)
+        S.selm_mg_vcycle(m.h, 0, v, b, cycle, 1)
+        out.append(v)
+    for cycle in (0, 31, 63):
+        want = [x.copy() for x in v0]
+        multigrid.vcycle(osys, 0, want, b0, philox.PhiloxNoise(11, 3, cycle), 1.0)
+        assert rel(from_dev(m.h, out[cycle]), want) < tol
