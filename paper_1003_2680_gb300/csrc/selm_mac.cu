@@ -1206,8 +1206,9 @@ selm_status zero_mean(selm_mac* h, cudaStream_t st) {
 // operator (FP32, selm_spectral.cu) as the preconditioner: exact up to FP32
 // rounding, so the FP64 recurrence gains about five digits per iteration
 // (64^3 + 8 rows to 1e-13: 3 iterations instead of 512, 0.59 ms instead of 18).
-// The residual and all inner products stay FP64.  *done = false when the
-// residual stops falling short of proj_tol.
+// The residual and all inner products stay FP64.  *done only with a residual
+// within proj_tol; false when it stops falling short of it, or is no number (r.z
+// of the largest fields overflows before r.r does).
 selm_status pressure_solve_spectral(selm_mac* h, const double* rhs, int* iters, double* resid, bool* done,
                                     cudaStream_t st) {
   const long long n = h->n_cells;
@@ -1233,7 +1234,7 @@ selm_status pressure_solve_spectral(selm_mac* h, const double* rhs, int* iters, 
   double rn = bn;
   int it = 0, idle = 0;
   *done = false;
-  while (bn > 0.0 && rn > tol * bn) {
+  while (bn > 0.0 && !(rn <= tol * bn)) {
     const int old = it & 1;   // r.z of this iteration in sc[old]
     MCK(precondition());
     {
@@ -1254,9 +1255,9 @@ selm_status pressure_solve_spectral(selm_mac* h, const double* rhs, int* iters, 
     MCK(cudaMemcpyAsync(h->host_sc, h->sc, 8 * sizeof(double), cudaMemcpyDeviceToHost, st));
     MCK(cudaStreamSynchronize(st));
     const double rn_new = std::sqrt(h->host_sc[3]);
-    idle = rn_new < 0.5 * rn ? 0 : idle + 1;   // (an iteration gains several digits; NaN counts as idle)
+    idle = rn_new < 0.5 * rn ? 0 : idle + 1;   // (an iteration gains several digits)
     rn = rn_new;
-    if (idle == 3) return SELM_OK;
+    if (idle == 3 || !std::isfinite(rn)) return SELM_OK;
   }
   *done = true;
   MRET(zero_mean(h, st));
@@ -1342,7 +1343,7 @@ selm_status pressure_solve(selm_mac* h, const double* rhs, int* iters, double* r
   MRET(zero_mean(h, st));
   if (iters) *iters = it;
   if (resid) *resid = bn > 0.0 ? rn / bn : 0.0;
-  if (bn > 0.0 && rn > tol * bn) {
+  if (bn > 0.0 && !(rn <= tol * bn)) {
     h->err = "pressure solve of the projection did not reach proj_tol";
     return SELM_ENOCONV;
   }

@@ -62,3 +62,29 @@ def test_stokes_velocity(S, n):
         torch.cuda.synchronize()
         S.selm_mg_destroy(h)
     assert ((us[0] - us[1]).norm() / us[0].norm()).item() <= 1e-9
+
+
+def test_projection_past_the_spectral_range(S):
+    """A field whose divergence has r.r within FP64 but r.S^-1 r beyond it: the
+    spectral preconditioner breaks down, and the projection falls back to the
+    diagonal one instead of returning what came out.  u = G phi + w with w free of
+    divergence, phi one mode along z (S^-1 of which is the largest): P~ u = w, to
+    proj_tol times the condition number (a few thousand)."""
+    n, K = 32, 8
+    h = S.selm_mac_create(S.make_mac_desc(3, n, K, projection=1))
+    nf, nc, fine = S.selm_mac_faces(h), S.selm_mac_cells(h), 2 * K * (2 * n) ** 2
+    z = torch.cat([(torch.arange(2 * K, device="cuda", dtype=torch.float64).repeat_interleave(4 * n * n) + 0.5) / (2 * n),
+                   (torch.arange(K, n, device="cuda", dtype=torch.float64).repeat_interleave(n * n) + 0.5) / n])
+    vol = torch.full((nc,), 1.0 / n ** 3, dtype=torch.float64, device="cuda")
+    vol[:fine] /= 8
+    g, w, div = (torch.empty(k, dtype=torch.float64, device="cuda") for k in (nf, nf, nc))
+    S.selm_mac_gradient(h, torch.cos(torch.pi * z), g)
+    S.selm_mac_project(h, torch.tensor(np.random.default_rng(3).standard_normal(nf), device="cuda"), w)
+    S.selm_mac_divergence(h, g + w, div)
+    rr = ((vol * div) ** 2).sum().item()
+    scale = 2.0 ** np.floor(0.5 * (np.log2(4e305) - np.log2(rr)))
+    out = torch.empty_like(w)
+    iters, res = S.selm_mac_project(h, (g + w) * scale, out)
+    assert iters > 16 and res <= 1e-13
+    assert ((out / scale - w).norm() / w.norm()).item() <= 1e-9
+    S.selm_mac_destroy(h)
