@@ -88,3 +88,44 @@ def test_projection_past_the_spectral_range(S):
     assert iters > 16 and res <= 1e-13
     assert ((out / scale - w).norm() / w.norm()).item() <= 1e-9
     S.selm_mac_destroy(h)
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("n,K", [(4, 2), (16, 3), (32, 0), (32, 9), (32, 32), (64, 0), (64, 8), (64, 64)])
+def test_projection_iterations(S, n, K, prec):
+    """The spectral solve preconditions conjugate gradients, which would hide a wrong
+    one behind more iterations or the diagonal fallback.  It is the operator's
+    inverse to about five digits (FP32), so 1e-12 takes at most 4 iterations: all
+    splits of rows, one to four rows per lane of the constant mode's scan and two
+    blocks of columns per row (n = 64).  The result is free of divergence to the
+    tolerance and is its own projection."""
+    h = S.selm_mac_create(S.make_mac_desc(3, n, K, projection=1, proj_tol=1e-12, precision=prec))
+    nf, nc, fine = S.selm_mac_faces(h), S.selm_mac_cells(h), 2 * K * (2 * n) ** 2
+    u = torch.tensor(np.random.default_rng(n + K).standard_normal(nf), device="cuda")
+    out, again = torch.empty_like(u), torch.empty_like(u)
+    div = torch.empty((2, nc), dtype=torch.float64, device="cuda")
+    iters, res = S.selm_mac_project(h, u, out)
+    assert iters <= 4 and res <= 1e-12
+    S.selm_mac_divergence(h, u, div[0])
+    S.selm_mac_divergence(h, out, div[1])
+    div[:, :fine] /= 8                                      # times the cells' volumes, as the solve measures it
+    assert (div[1].norm() / div[0].norm()).item() <= 1e-11
+    S.selm_mac_project(h, out, again)
+    assert ((again - out).norm() / out.norm()).item() <= 1e-10
+    S.selm_mac_destroy(h)
+
+
+@pytest.mark.parametrize("n", [64, 128])
+def test_stokes_velocity_of_large_grids(S, n):
+    """test_stokes_velocity's comparison up to the largest grid of the spectral solve
+    (FP64 handle: FAC), to 1e-9 from solves to 1e-11."""
+    us = []
+    for prec in (0, 1):
+        h = S.selm_mg_create(S.make_desc(dim=3, n=n, mu=0.9, precision=prec, tol=1e-11))
+        f = torch.tensor(np.random.default_rng(n).standard_normal(S.selm_mg_layout(h, 0, 0, 0)[2]), device="cuda")
+        u = torch.empty_like(f)
+        assert S.selm_mg_stokes_solve(h, f, u)[1] <= 1e-11
+        us.append(u)
+        torch.cuda.synchronize()
+        S.selm_mg_destroy(h)
+    assert ((us[0] - us[1]).norm() / us[0].norm()).item() <= 1e-9
