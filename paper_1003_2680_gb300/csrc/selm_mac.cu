@@ -1413,6 +1413,44 @@ selm_status spread(selm_mac* h, int np, const double* X, const double* F, double
   return SELM_OK;
 }
 
+// The buffers of k_draw's normals: a level's for every sweep of its V-cycle, the
+// slab's for every patch sweep.  SELM_ENOMEM leaves the handle without them.
+selm_status alloc_drawn(selm_mac* h, int levels, cudaStream_t st) {
+  const int sweeps = h->d.nu_pre + h->d.nu_post;
+  long long normals = 0;
+  for (int l = 0; l + 1 < levels; ++l) normals += (long long)h->lev[l].cls.npos * sweeps;
+  if (!h->pstart.empty()) normals += (long long)h->Apatch.npos * h->d.nu_patch;
+  double* base = nullptr;
+  if (normals <= 0) return SELM_OK;
+  if (cudaMalloc((void**)&base, normals * sizeof(double)) != cudaSuccess) {
+    cudaGetLastError();
+    return SELM_ENOMEM;
+  }
+  h->allocs.push_back(base);
+  DrawLists D{};
+  auto add = [&](const SellDev& S, const std::vector<int>& starts, int n, int level1, bool slab) -> selm_status {
+    DrawList& q = D.l[D.n++];
+    q.first = D.total;
+    q.npos = S.npos;
+    q.sweeps = n;
+    q.sweep0 = 0;
+    q.level1 = level1;
+    q.slab = slab ? 1 : 0;
+    q.ncol = (int)starts.size();
+    q.row = S.row;
+    q.out = base;
+    base += (long long)S.npos * n;
+    D.total += (long long)n * (slab ? S.npos : S.npos / 2);
+    return upload(h, starts, &q.cstart, st);
+  };
+  for (int l = 0; l + 1 < levels; ++l) MRET(add(h->lev[l].cls, h->lev[l].cstart, sweeps, l + 1, false));
+  if (!h->pstart.empty()) MRET(add(h->Apatch, h->pstart, h->d.nu_patch, 0, true));
+  for (int l = 0; l + 1 < levels; ++l) h->lev[l].drawn = D.l[l].out;
+  if (!h->pstart.empty()) h->drawn_patch = D.l[D.n - 1].out;
+  h->draws = D;
+  return SELM_OK;
+}
+
 std::string fill_defaults(selm_mac_desc* d) {
   if (d->mu == 0.0) d->mu = 1.0;
   if (d->nu_pre == 0) d->nu_pre = 2;
@@ -1580,37 +1618,6 @@ selm_status selm_mac_create(const selm_mac_desc* desc, void* stream, selm_mac** 
     }
     CREATE_STEP(upload_sell(h, make_sell(Et, natural_order(Et.nr), false), false, &h->Et, st));
   }
-  if (!f32 && plan.levels < kDrawLists) {   // buffers of the normals; without memory for them the rows draw
-    long long normals = 0;
-    for (int l = 0; l + 1 < plan.levels; ++l) normals += (long long)h->lev[l].cls.npos * (d.nu_pre + d.nu_post);
-    if (!h->pstart.empty()) normals += (long long)h->Apatch.npos * d.nu_patch;
-    double* base = nullptr;
-    if (normals > 0 && cudaMalloc((void**)&base, normals * sizeof(double)) == cudaSuccess) {
-      h->allocs.push_back(base);
-      auto add = [&](const SellDev& S, const std::vector<int>& starts, int sweeps, int level1, bool slab,
-                     double** out) -> selm_status {
-        if (sweeps <= 0) return SELM_OK;
-        DrawList& q = h->draws.l[h->draws.n++];
-        q.first = h->draws.total;
-        q.npos = S.npos;
-        q.sweeps = sweeps;
-        q.sweep0 = 0;
-        q.level1 = level1;
-        q.slab = slab ? 1 : 0;
-        q.ncol = (int)starts.size();
-        q.row = S.row;
-        q.out = base;
-        *out = base;
-        base += (long long)S.npos * sweeps;
-        h->draws.total += (long long)sweeps * (slab ? S.npos : S.npos / 2);
-        return upload(h, starts, &q.cstart, st);
-      };
-      for (int l = 0; l + 1 < plan.levels; ++l)
-        CREATE_STEP(add(h->lev[l].cls, h->lev[l].cstart, d.nu_pre + d.nu_post, l + 1, false, &h->lev[l].drawn));
-      if (!h->pstart.empty()) CREATE_STEP(add(h->Apatch, h->pstart, d.nu_patch, 0, true, &h->drawn_patch));
-    }
-    cudaGetLastError();
-  }
   // the uniform fine lattice of the particle kernel
   h->fine.level = 0;
   h->fine.ncomp = plan.fine_ncomp;
@@ -1640,11 +1647,6 @@ selm_status selm_mac_create(const selm_mac_desc* desc, void* stream, selm_mac** 
   h->fw2 = (double*)p;
   CREATE_STEP(alloc(h, (size_t)plan.fine_size * 8, &p, st));
   h->fine_buf = (double*)p;
-  if (mac_spectral_supported(d.dim, d.n, d.K) && cudaMalloc(&h->spec, mac_spectral_bytes(d.n, d.K)) == cudaSuccess)
-    h->allocs.push_back(h->spec);
-  else
-    h->spec = nullptr;   // another grid, or no memory for the spectra
-  cudaGetLastError();
   for (double** b : {&h->cg_x, &h->cg_r, &h->cg_z, &h->cg_p, &h->cg_q, &h->pv}) {
     CREATE_STEP(alloc(h, (size_t)nc * 8, &p, st));
     *b = (double*)p;
@@ -1670,6 +1672,21 @@ selm_status selm_mac_create(const selm_mac_desc* desc, void* stream, selm_mac** 
     cudaGetLastError();
     h->cap = nullptr;
     h->graphs = false;
+  }
+  // What the handle can do without comes last, so that it takes no memory from
+  // what it needs: the spectra of the pressure solve (else the diagonal
+  // preconditioner) and the drawn normals of FP64 cycles (else the rows draw).
+  if (mac_spectral_supported(d.dim, d.n, d.K) && cudaMalloc(&h->spec, mac_spectral_bytes(d.n, d.K)) == cudaSuccess)
+    h->allocs.push_back(h->spec);
+  else
+    h->spec = nullptr;
+  cudaGetLastError();
+  if (!f32 && plan.levels < kDrawLists) {
+    r = alloc_drawn(h, plan.levels, st);
+    if (r == SELM_ENOMEM)
+      h->err.clear();
+    else if (r != SELM_OK)
+      return fail(r);
   }
   if (cudaStreamSynchronize(st) != cudaSuccess) {
     h->err = "set-up copies failed";

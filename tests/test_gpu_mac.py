@@ -315,3 +315,30 @@ def test_benchmark_size_properties(S):
         assert ((Az - b).norm() / b.norm()).item() < 2e-10
     finally:
         S.selm_mac_destroy(h)
+
+
+def test_create_without_memory_for_the_optional_buffers(S):
+    """The buffers of drawn normals (and the spectra) come after everything the handle
+    needs: with 100 MB less than all of it free, which is less than the normals of
+    60 sweeps and more than the allocations that follow their old place, create
+    succeeds and the chain is the same."""
+    desc = S.make_mac_desc(3, 64, 16, precision=S.SELM_FP64, nu_pre=30, nu_post=30, projection=1, seed=5)
+    xi = []
+    left = None
+    for _ in range(2):
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        hog = None
+        if left is not None:
+            hog = torch.empty(torch.cuda.mem_get_info()[0] - left, dtype=torch.uint8, device="cuda")
+        free = torch.cuda.mem_get_info()[0]
+        h = S.selm_mac_create(desc)
+        if left is None:
+            left = free - torch.cuda.mem_get_info()[0] - 100 * 2 ** 20
+        del hog
+        torch.cuda.empty_cache()
+        xi.append(torch.empty(S.selm_mac_faces(h), dtype=torch.float64, device="cuda"))
+        S.selm_mac_sample(h, 1, xi[-1])
+        torch.cuda.synchronize()
+        S.selm_mac_destroy(h)
+    assert xi[0].any() and torch.equal(xi[0], xi[1])
