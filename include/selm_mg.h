@@ -173,14 +173,14 @@ enum {
    first level whose slabs fit in shared memory); the levels above it run as
    GPU-wide launches.  Re-plans both systems' engines.
    SELM_OPT_LEVEL_COOP (default 1): each half V-cycle of a level above the
-   engine runs as one cooperative launch over every SM (FP32 levels in 2-D, and
-   of more than a million unknowns in 3-D, as launches of two colours each, with
-   the cooperative form's values).  1: with FP32 inner
+   engine runs as one cooperative launch over every SM.  1: with FP32 inner
    cycles the colour passes run in dataflow order, each site update waiting
    for its coupled neighbours only (each stored value carries the parity of
    its update count in its least significant mantissa bit, at most 1 ulp from
    the rounded update); FP64 levels, and levels whose stencil admits no such
-   order, separate the passes by grid barriers.  2: grid barriers always.
+   order, separate the passes by grid barriers.  FP32 levels in 2-D, and of more
+   than a million unknowns in 3-D, run as launches of two colours each instead,
+   with the same values.  2: cooperative launches with grid barriers, always.
    Every wait is bounded; a timed-out wait is reported as SELM_ECUDA by the
    next solve's norm read.  0 selects launches per colour pass.  All give
    the same result up to rounding. */

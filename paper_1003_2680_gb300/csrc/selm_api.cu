@@ -296,9 +296,11 @@ selm_status vcycle_t(selm_mg* h, Sys& s, int l, T* v0, const T* b0, bool noise, 
   //    costs about 3 us of update latency plus its sites over 78 K threads (64^3: 446
   //    cooperative, 473 with launches; 72^3: 854 and 684; 80^3: 849 and 743).
   // Launches for a level in dataflow order store the same parity bits, so both
-  // forms give the same values.
+  // forms give the same values.  SELM_OPT_LEVEL_COOP = 2 keeps the cooperative form
+  // (grid barriers) on every level.
   const bool flow_level = sizeof(T) == 4 && s.coop_flow && L.flow;
-  const bool full_passes = coarse_row_pairs<T>(L) && (L.c[0].ny == 1 || (flow_level && L.size > 1000000));
+  const bool full_passes =
+      s.coop_flow && coarse_row_pairs<T>(L) && (L.c[0].ny == 1 || (flow_level && L.size > 1000000));
   const bool coop = l > 0 && !last && !L.rb && level_sites(L) <= kCoopMaxSites && s.use_engine && s.use_coop &&
                     eng.valid && l < eng.params.l0 && s.coop_bar && level_coop_supported<T>(L);
   const bool tags = coop && full_passes && flow_level;

@@ -120,3 +120,32 @@ def test_normals_drawn_into_another_block(dim, n, prec):
         want = [x.copy() for x in v0]
         multigrid.vcycle(osys, 0, want, b0, philox.PhiloxNoise(11, 3, cycle), 1.0)
         assert rel(from_dev(m.h, out[cycle]), want) < tol
+
+
+@pytest.mark.parametrize("dim,n", [(2, 768), (2, 160), (3, 144)])
+@pytest.mark.parametrize("noise", [0, 1])
+def test_grid_barriers_on_request(dim, n, noise):
+    """SELM_OPT_LEVEL_COOP = 2: level 1 as two cooperative launches, also where the
+    default takes row-pair launches (as many launches as without the option, less the
+    memory operations).  2-D levels admit no dataflow order, so there the default
+    stores no parity bits and gives the cooperative form's values bit by bit; in 3-D
+    it does, within the FP32 tolerance."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1003_2680_gb300 import selm as S
+    m = S.SelmMG(dim=dim, n=n, precision=1, seed=11, instance=3)
+    b = torch.randn(comps(m.h, 0, 0)[1], device="cuda", generator=torch.Generator("cuda").manual_seed(5))
+    out, launches = {}, {}
+    for coop in (0, 1, 2):
+        S.selm_mg_set_option(m.h, S.SELM_OPT_LEVEL_COOP, coop)
+        S.selm_mg_set_option(m.h, S.SELM_OPT_ENGINE_LEVEL, 2)
+        v = torch.zeros_like(b)
+        before = S.selm_kernel_launches()
+        S.selm_mg_vcycle(m.h, 0, v, b, 7, noise)
+        launches[coop] = S.selm_kernel_launches() - before
+        out[coop] = v
+    # level 1: 6 class pairs (3-D; 3 in 2-D) x 4 sweeps, residual, restriction, prolongation, against 2
+    assert launches[0] == launches[1] == launches[2] + (24 if dim == 3 else 12) + 1
+    if dim == 2:
+        assert torch.equal(out[1], out[2])
+    assert ((out[1] - out[2]).norm() / out[2].norm()).item() < 1e-5
