@@ -169,9 +169,12 @@ enum {
 /* SELM_OPT_ENGINE_CLUSTER: largest thread-block cluster the coarse engine may
    use (1..16; 0 = the largest that fits).  Re-plans the engine; synchronises
    the legacy default stream.
-   SELM_OPT_ENGINE_LEVEL: first level the coarse engine may take (0 = the
-   first level whose slabs fit in shared memory); the levels above it run as
-   GPU-wide launches.  Re-plans both systems' engines.
+   SELM_OPT_ENGINE_LEVEL: first level the coarse engine may take, which it does
+   if its slabs fit in shared memory (else the first one below whose slabs do);
+   the levels above it run as GPU-wide launches.  0: the library's choice, which
+   leaves levels that pay over the whole GPU to cooperative launches (level 1 from
+   2^17 sites per component; in FP64 every level of more than 2^15).  Re-plans both
+   systems' engines.
    SELM_OPT_LEVEL_COOP (default 1): each half V-cycle of a level above the
    engine runs as one cooperative launch over every SM.  1: with FP32 inner
    cycles the colour passes run in dataflow order, each site update waiting

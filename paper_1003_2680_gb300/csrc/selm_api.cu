@@ -623,13 +623,15 @@ namespace {
 // with the cooperative launches (a pass of a 40^3 level: about 12 us in a
 // cluster, 6 us over the GPU; of a 20^3 level: 3.4 and 5 us).
 int engine_first_level(const selm_mg* h, const Sys& s) {
+  if (s.engine_level > 0) return s.engine_level;
   auto coop = [&](int l) {
     return h->esize == 4 ? level_coop_supported<float>(s.lev[l]) : level_coop_supported<double>(s.lev[l]);
   };
-  int first = s.engine_level > 0 ? s.engine_level : 1;
-  if (s.engine_level <= 0 && s.use_coop && s.levels >= 4 && level_sites(s.lev[1]) >= (1ll << 17) && coop(1)) first = 2;
-  while (h->esize == 8 && s.use_coop && first + 2 < s.levels && !s.lev[first].rb &&
-         level_sites(s.lev[first]) > (1ll << 15) && level_sites(s.lev[first]) <= kCoopMaxSites && coop(first))
+  int first = 1;
+  if (!s.use_coop) return first;
+  if (s.levels >= 4 && level_sites(s.lev[1]) >= (1ll << 17) && coop(1)) first = 2;
+  while (h->esize == 8 && first + 2 < s.levels && !s.lev[first].rb && level_sites(s.lev[first]) > (1ll << 15) &&
+         level_sites(s.lev[first]) <= kCoopMaxSites && coop(first))
     ++first;
   return first;
 }

@@ -149,3 +149,25 @@ def test_grid_barriers_on_request(dim, n, noise):
     if dim == 2:
         assert torch.equal(out[1], out[2])
     assert ((out[1] - out[2]).norm() / out[2].norm()).item() < 1e-5
+
+
+@pytest.mark.parametrize("dim,n", [(3, 80), (2, 512)])
+def test_engine_level_on_request(dim, n):
+    """SELM_OPT_ENGINE_LEVEL on an FP64 handle: the engine starts at the level asked
+    for (40^3, 256^2: levels that the library's own choice leaves to cooperative
+    launches), with the same V-cycle to 1e-12."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1003_2680_gb300 import selm as S
+    m = S.SelmMG(dim=dim, n=n, precision=0, seed=11, instance=3)
+    b = torch.randn(comps(m.h, 0, 0)[1], device="cuda", dtype=torch.float64,
+                    generator=torch.Generator("cuda").manual_seed(5))
+    assert S.selm_mg_engine_info(m.h)[0] == 2
+    out = []
+    for level in (0, 1):
+        S.selm_mg_set_option(m.h, S.SELM_OPT_ENGINE_LEVEL, level)
+        assert S.selm_mg_engine_info(m.h)[0] == (level or 2)
+        v = torch.zeros_like(b)
+        S.selm_mg_vcycle(m.h, 0, v, b, 7, 1)
+        out.append(v)
+    assert ((out[0] - out[1]).norm() / out[1].norm()).item() < 1e-12
