@@ -376,16 +376,17 @@ __device__ __forceinline__ long long fx_align(long long bits, int emax) {
   return d >= 63 ? (m < 0 ? -1ll : 0ll) : ((m * 32) >> d);
 }
 
-// The same for a window of exponents within 31 of emax (none zero), one 64-bit
-// shift by less than 32, the magnitude truncated; the caller adds neg.
-__device__ __forceinline__ unsigned long long fx_align31(long long bits, unsigned emax20, unsigned* neg) {
+// The same for a window of exponents within 31 of emax (none zero): one 64-bit
+// shift by less than 32.  A negative value -a is ~((a - 1) >> d), the same floor.
+__device__ __forceinline__ unsigned long long fx_align31(long long bits, unsigned emax20) {
   const unsigned hi = (unsigned)((unsigned long long)bits >> 32), lo = (unsigned)bits;
   const unsigned sh = (emax20 - (hi & 0x7ff00000u)) >> 20;
   const unsigned mh = (hi & 0x000fffffu) | 0x00100000u;
-  const unsigned h5 = __funnelshift_l(lo, mh, 5), l5 = lo << 5;
-  const unsigned s = (unsigned)((int)hi >> 31);   // all ones for a negative value
-  *neg = s;
-  return ((unsigned long long)((h5 >> sh) ^ s) << 32) | (__funnelshift_r(l5, h5, sh) ^ s);
+  const int s = (int)hi >> 31;   // all ones for a negative value
+  const unsigned long long a =
+      (((unsigned long long)__funnelshift_l(lo, mh, 5) << 32) | (lo << 5)) + (unsigned long long)(long long)s;
+  const unsigned ah = (unsigned)(a >> 32), al = (unsigned)a;
+  return ((unsigned long long)((ah >> sh) ^ (unsigned)s) << 32) | (__funnelshift_r(al, ah, sh) ^ (unsigned)s);
 }
 
 // S 2^e2 rounded to nearest even as FP64 (S != 0 and the result normal,
@@ -494,23 +495,16 @@ __global__ void __launch_bounds__(kFxBlock, 5) k_outer_residual_fx(LevelDev L, R
       // S = the neighbours' sum, C = the centre
       unsigned long long S[4], C[4];
       if (emin20 != 0u && emax20 - emin20 <= (31u << 20)) {
-        unsigned n[22];
         unsigned long long Z[22];
 #pragma unroll
-        for (int q = 0; q < 22; ++q) Z[q] = fx_align31(w[q], emax20, &n[q]);
+        for (int q = 0; q < 22; ++q) Z[q] = fx_align31(w[q], emax20);
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          C[e] = Z[e] - (long long)(int)n[e];
-          const int l = e == 0 ? 4 : e - 1, r = e == 3 ? 5 : e + 1;
-          S[e] = Z[l] + Z[r];
-          int neg = (int)n[l] + (int)n[r];
+          C[e] = Z[e];
+          S[e] = Z[e == 0 ? 4 : e - 1] + Z[e == 3 ? 5 : e + 1];
 #pragma unroll
           for (int q = 0; q < 4; ++q)
-            if (present[q]) {
-              S[e] += Z[6 + 4 * q + e];
-              neg += (int)n[6 + 4 * q + e];
-            }
-          S[e] -= (long long)neg;
+            if (present[q]) S[e] += Z[6 + 4 * q + e];
         }
       } else {
 #pragma unroll

@@ -171,3 +171,53 @@ def test_engine_level_on_request(dim, n):
         S.selm_mg_vcycle(m.h, 0, v, b, 7, 1)
         out.append(v)
     assert ((out[0] - out[1]).norm() / out[1].norm()).item() < 1e-12
+
+
+@pytest.mark.parametrize("span,zeros", [(0, False), (20, False), (31, False), (40, False), (70, False), (20, True)])
+def test_fixed_point_residual_rounding(span, zeros):
+    """The FP32 outer residual's integer sum, bit by bit: every value of a window
+    (4 sites of a row, their neighbours) becomes floor(z 2^(1080 - emax)), emax the
+    window's largest exponent, whatever the spread of the exponents (up to 31 bits
+    and beyond are separate code) and the signs.  b = s RN(sum), so any other
+    rounding of a value leaves a residual: r = 0 exactly."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import math
+    from fractions import Fraction
+
+    import numpy as np
+    from paper_1003_2680_gb300 import selm as S
+    n = 8
+    m = S.SelmMG(dim=3, n=n, precision=1, seed=11)
+    lay, size = comps(m.h, 0, 0)
+    rng = np.random.default_rng(span)
+    z = rng.choice([-1.0, 1.0], size) * rng.uniform(0.5, 1.0, size) * 2.0 ** rng.integers(-span, 1, size)
+    if zeros:
+        z[rng.random(size) < 0.05] = 0.0
+    r = torch.empty(size, dtype=torch.float32, device="cuda")
+    probe = np.zeros(size)
+    (nz, ny, nx), off = lay[0]
+    centre = off + (3 * ny + 3) * nx + 3
+    probe[centre] = 1.0
+    S.selm_mg_outer_residual(m.h, 0, torch.tensor(probe, device="cuda"), torch.zeros(size, dtype=torch.float64, device="cuda"), r)
+    s = -r[centre].item() / 6
+    assert s > 0 and math.frexp(s)[0] == 0.5          # a power of two: s RN(sum) is exact
+    b = np.zeros(size)
+    for ci, ((nz, ny, nx), off) in enumerate(lay):
+        f = z[off:off + nz * ny * nx].reshape(nz, ny, nx)
+        g = b[off:off + nz * ny * nx].reshape(nz, ny, nx)
+        for k in range(nz):
+            dg = 6 + ((k == 0) + (k == nz - 1) if ci < 2 else 0)      # no-slip ghost on cell centres
+            for j in range(ny):
+                rows = [f[k, j - 1], f[k, (j + 1) % ny]] + ([f[k - 1, j]] if k > 0 else []) + ([f[k + 1, j]] if k + 1 < nz else [])
+                for x0 in range(0, nx, 4):
+                    own = f[k, j].take(range(x0 - 1, x0 + 5), mode="wrap")
+                    win = np.concatenate([own] + [q[x0:x0 + 4] for q in rows])
+                    emax = max(math.frexp(v)[1] for v in win if v != 0.0) + 1022    # biased exponent
+                    fix = lambda v: math.floor(Fraction(v) * Fraction(2) ** (1080 - emax))
+                    for e in range(4):
+                        t = dg * fix(own[1 + e]) - fix(own[e]) - fix(own[2 + e]) - sum(fix(q[x0 + e]) for q in rows)
+                        g[k, j, x0 + e] = s * float(Fraction(t) * Fraction(2) ** (emax - 1080))
+    norm = torch.zeros(1, dtype=torch.float64, device="cuda")
+    S.selm_mg_outer_residual(m.h, 0, torch.tensor(z, device="cuda"), torch.tensor(b, device="cuda"), r, norm)
+    assert not r.any() and norm.item() == 0.0
