@@ -618,7 +618,8 @@ namespace {
 // level 1 goes to cooperative launches when it is large (a pass of level 1
 // then spreads over every SM instead of one cluster per component, which
 // pays once a component holds 2^17 sites or more) and the engine starts at
-// level 2; otherwise the engine takes every level from 1.
+// level 2; otherwise the engine takes every level from 1 (from engine_min, where
+// that is set).
 // FP64: the FP64 pipe bounds a pass, so levels of more than 2^15 sites stay
 // with the cooperative launches (a pass of a 40^3 level: about 12 us in a
 // cluster, 6 us over the GPU; of a 20^3 level: 3.4 and 5 us).
@@ -627,9 +628,9 @@ int engine_first_level(const selm_mg* h, const Sys& s) {
   auto coop = [&](int l) {
     return h->esize == 4 ? level_coop_supported<float>(s.lev[l]) : level_coop_supported<double>(s.lev[l]);
   };
-  int first = 1;
+  int first = s.engine_min > 0 ? s.engine_min : 1;
   if (!s.use_coop) return first;
-  if (s.levels >= 4 && level_sites(s.lev[1]) >= (1ll << 17) && coop(1)) first = 2;
+  if (s.engine_min <= 0 && s.levels >= 4 && level_sites(s.lev[1]) >= (1ll << 17) && coop(1)) first = 2;
   while (h->esize == 8 && first + 2 < s.levels && !s.lev[first].rb && level_sites(s.lev[first]) > (1ll << 15) &&
          level_sites(s.lev[first]) <= kCoopMaxSites && coop(first))
     ++first;
@@ -657,7 +658,7 @@ size_t footprint_with_host(const selm_mg_desc& d, const HostSystem& host, size_t
   return p.lay.total;
 }
 
-selm_status create_with_host(const selm_mg_desc& d, const HostSystem& host, int engine_level, bool use_coop,
+selm_status create_with_host(const selm_mg_desc& d, const HostSystem& host, int engine_min, bool use_coop,
                              int rb_level, size_t extra_bytes, cudaStream_t st, selm_mg** out, size_t* extra_off) {
   *out = nullptr;
   selm_mg* h = new (std::nothrow) selm_mg();
@@ -670,7 +671,7 @@ selm_status create_with_host(const selm_mg_desc& d, const HostSystem& host, int 
   h->esize = d.precision == SELM_FP64 ? 8 : 4;
   h->key.k0 = (uint32_t)(d.seed & 0xffffffffu) ^ (uint32_t)(d.instance >> 32);
   h->key.k1 = (uint32_t)(d.seed >> 32) ^ (uint32_t)(d.instance & 0xffffffffu);
-  h->vel.engine_level = engine_level;
+  h->vel.engine_min = engine_min;
   h->vel.use_coop = use_coop;
   Plan p;
   make_plan(d, h->vel, nullptr, h->esize, &p, true);

@@ -25,7 +25,8 @@ struct Sys {
   EnginePlanT<double> engd;   // (FP64 inner)
   bool use_engine = true;
   int engine_cluster = 0;     // preferred cluster size of the engine (0 = largest that fits)
-  int engine_level = 0;       // first level the engine may take (0 = the first that fits)
+  int engine_level = 0;       // first level of the engine as the caller's option gives it (0 = the library's choice)
+  int engine_min = 0;         // earliest level of the library's choice (0 = level 1)
   void* eng_dev = nullptr;    // device slot of the engine plan
   bool use_coop = true;       // levels above the engine: cooperative launches (else one per pass)
   bool coop_flow = true;      // FP32 cooperative passes in dataflow order where the level allows it
@@ -143,8 +144,8 @@ selm_status replan_engine(selm_mg* h, int cluster, cudaStream_t st);
 // A handle around a prepared host hierarchy (one system, no projection), with
 // V-cycle scratch only plus `extra_bytes` of workspace for the caller at
 // *extra_off.  Level rb_level (if >= 0) is smoothed red-black; the engine
-// starts at engine_level at the earliest.  The composite form builds on it.
-selm_status create_with_host(const selm_mg_desc& d, const HostSystem& host, int engine_level, bool use_coop,
+// starts at engine_min at the earliest.  The composite form builds on it.
+selm_status create_with_host(const selm_mg_desc& d, const HostSystem& host, int engine_min, bool use_coop,
                              int rb_level, size_t extra_bytes, cudaStream_t st, selm_mg** out, size_t* extra_off);
 size_t footprint_with_host(const selm_mg_desc& d, const HostSystem& host, size_t extra_bytes);
 // One V-cycle (Algorithm 3) of system s from `level` down, on the internal

@@ -319,3 +319,20 @@ def test_outer_update_widens_exactly(S):
     z = torch.zeros(size, dtype=torch.float64, device="cuda")
     selm.selm_mg_outer_update(m.h, 0, z, d)
     assert torch.equal(z, d.double())
+
+
+def test_large_fp64_levels_stay_cooperative(S):
+    """The first Galerkin level below the base is 40^3 (64000 sites) at n = 80 and
+    24^3 at n = 48: in FP64 the former runs as two cooperative launches a cycle in
+    front of the engine, which takes the latter itself."""
+    launches = []
+    for n, K in ((80, 9), (48, 6)):
+        c, _ = handle(S, 3, n, K, "fp64", ncomp=1)
+        z = torch.zeros(S.selm_comp_size(c), dtype=torch.float64, device="cuda")
+        b = torch.ones_like(z)
+        before = S.selm_kernel_launches()
+        S.selm_comp_fac_cycle(c, z, b, 0, 0)
+        launches.append(S.selm_kernel_launches() - before)
+        torch.cuda.synchronize()
+        S.selm_comp_destroy(c)
+    assert launches[0] == launches[1] + 2
