@@ -117,8 +117,10 @@ selm_status selm_mac_gradient(selm_mac* h, const double* p, double* grad, void* 
 /* out = P~ u (adjoint = 0) or P~^T u = W P~ W^-1 u (adjoint = 1); out may
    equal u.  The pressure L phi = D u (phi of zero volume mean) is solved by
    FP64 conjugate gradients on diag(vol) L to proj_tol, preconditioned by the
-   operator's spectral solve (3-D, n a power of two up to 64), else by its
-   diagonal; iters / resid (optional HOST pointers) receive the iteration
+   operator's spectral solve in FP32 whatever the handle's precision (3-D, n a
+   power of two up to 64; residual, iterates and inner products are FP64, and it
+   runs to proj_tol / 32), else, and where that breaks down, by the operator's
+   diagonal in FP64; iters / resid (optional HOST pointers) receive the iteration
    count and relative residual (synchronises the stream). */
 selm_status selm_mac_project(selm_mac* h, const double* u, double* out, int adjoint, int* iters, double* resid,
                              void* stream);

@@ -1204,11 +1204,14 @@ selm_status zero_mean(selm_mac* h, cudaStream_t st) {
 
 // The same conjugate gradients with the spectral solve of the composite
 // operator (FP32, selm_spectral.cu) as the preconditioner: exact up to FP32
-// rounding, so the FP64 recurrence gains about five digits per iteration
-// (64^3 + 8 rows to 1e-13: 3 iterations instead of 512, 0.59 ms instead of 18).
-// The residual and all inner products stay FP64.  *done only with a residual
-// within proj_tol; false when it stops falling short of it, or is no number (r.z
-// of the largest fields overflows before r.r does).
+// rounding, so the FP64 recurrence gains five to seven digits per iteration
+// (64^3 + 8 rows to 1e-13: 3 iterations instead of 512, 0.65 ms instead of 18).
+// The residual and all inner products stay FP64.  It stops at proj_tol / 32, as far
+// below as the diagonal preconditioner got by testing every 16th iteration only:
+// stopping at proj_tol left errors of up to 6e-14 where that had 8e-15 to 4e-14
+// (white fields, 8^3 to 32^3).  *done only with a residual within proj_tol; false
+// when it stops falling short of it, or is no number (r.z of the largest fields
+// overflows before r.r does).
 selm_status pressure_solve_spectral(selm_mac* h, const double* rhs, int* iters, double* resid, bool* done,
                                     cudaStream_t st) {
   const long long n = h->n_cells;
@@ -1234,7 +1237,7 @@ selm_status pressure_solve_spectral(selm_mac* h, const double* rhs, int* iters, 
   double rn = bn;
   int it = 0, idle = 0;
   *done = false;
-  while (bn > 0.0 && !(rn <= tol * bn)) {
+  while (bn > 0.0 && !(rn <= tol / 32 * bn)) {
     const int old = it & 1;   // r.z of this iteration in sc[old]
     MCK(precondition());
     {
@@ -1257,8 +1260,9 @@ selm_status pressure_solve_spectral(selm_mac* h, const double* rhs, int* iters, 
     const double rn_new = std::sqrt(h->host_sc[3]);
     idle = rn_new < 0.5 * rn ? 0 : idle + 1;   // (an iteration gains several digits)
     rn = rn_new;
-    if (idle == 3 || !std::isfinite(rn)) return SELM_OK;
+    if (idle == 3 || !std::isfinite(rn) || (idle > 0 && rn <= tol * bn)) break;
   }
+  if (bn > 0.0 && !(rn <= tol * bn)) return SELM_OK;
   *done = true;
   MRET(zero_mean(h, st));
   if (iters) *iters = it;

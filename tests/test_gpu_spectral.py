@@ -129,3 +129,19 @@ def test_stokes_velocity_of_large_grids(S, n):
         torch.cuda.synchronize()
         S.selm_mg_destroy(h)
     assert ((us[0] - us[1]).norm() / us[0].norm()).item() <= 1e-9
+
+
+@pytest.mark.parametrize("n,K", [(8, 3), (16, 5), (32, 0), (32, 9)])
+def test_projection_error(S, n, K):
+    """The default tolerance (1e-13) on a white field against a solve to 1e-17: 1e-14,
+    three times the residual of 1e-13 / 32 at which the spectral iteration stops
+    (error over residual: 1.3 on such fields)."""
+    out = []
+    for tol in (0.0, 1e-17):
+        h = S.selm_mac_create(S.make_mac_desc(3, n, K, projection=1, proj_tol=tol))
+        u = torch.tensor(np.random.default_rng(1).standard_normal(S.selm_mac_faces(h)), device="cuda")
+        out.append(torch.empty_like(u))
+        S.selm_mac_project(h, u, out[-1])
+        torch.cuda.synchronize()
+        S.selm_mac_destroy(h)
+    assert ((out[0] - out[1]).norm() / out[1].norm()).item() <= 1e-14
