@@ -322,7 +322,9 @@ selm_status selm_batch_step(selm_batch* b, const int* np, double* const* X, cons
    persistent form (see selm_batch_set_persistent) and for engine cluster sizes
    16, 8 and 4 of the graph form, keeps the best shape of each and runs the
    faster form from then on (selm_batch_info tells which); *chosen_cluster
-   receives the graph form's cluster size. */
+   receives the graph form's cluster size.  Cluster sizes that would move a level
+   of some system out of its engine are passed over: its values would round
+   differently. */
 selm_status selm_batch_autotune(selm_batch* b, int* chosen_cluster, void* stream);
 enum { SELM_BATCH_SOLVE = 0, SELM_BATCH_SAMPLE = 1 };
 /* One FAC cycle (Algorithm 1) of every system of the batch, the systems side

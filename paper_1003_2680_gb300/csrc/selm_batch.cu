@@ -581,6 +581,8 @@ selm_status selm_batch_autotune(selm_batch* b, int* chosen_cluster, void* stream
   // A cluster too small for a level that the first candidate's engine holds is
   // passed over: the level would run as per-pass launches, whose FP32 sums round
   // differently, and the tuned batch would depend on the timing in its last bits.
+  // The price, for batches with 96^3 systems (48^3 leaves clusters of 4): 64 systems
+  // of 32^3 to 128^3 take 66.7 ms a step with clusters of 8, 61.5 with 4.
   b->persistent = false;
   const int cands[3] = {16, 8, 4};
   std::vector<int> first_level(b->n, -1);

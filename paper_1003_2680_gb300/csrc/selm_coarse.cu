@@ -24,13 +24,14 @@
 // sit in registers, all of a site's loads are issued before the first sum,
 // everything about a site but the values v is loaded off the critical path,
 // the normals of a noisy launch are drawn once at its start, and the coarsest
-// step is spread over the cluster.  64^3 velocity V-cycle (levels of 32^3 and
-// below), one launch: 157 -> 121 us, noisy 211 -> 150 us; 48^3: 125 -> 90,
-// noisy 184 -> 107 us; 96^3: 235 -> 204, noisy 353 -> 272 us.  Where the 121 us
-// go: 48 passes of 32^3 at 0.8 us, of 16^3 at 0.7 us, of 8^3 at 0.3 us, the
-// coarsest step 5 us, transfers 17 us, staging 5 us.
+// step is spread over the cluster.  One launch by events, before and after: 48^3
+// (levels of 24^3 and below) 152 -> 95 us, noisy 215 -> 112; 64^3 162 -> 127, noisy
+// 214 -> 156; 96^3 331 -> 207, noisy 425 -> 273; in FP64 64^2 185 -> 107, noisy
+// 403 -> 137, and 48^3 634 -> 408, noisy 1015 -> 493.  Where 64^3's go, noise-free:
+// 48 passes of 32^3 at 0.8 us, of 16^3 at 0.7 us, of 8^3 at 0.3 us, the coarsest
+// step 5 us, transfers 17 us, staging 5 us.
 // The 2-D and 3-D forms are separate kernels: as branches of one kernel their
-// code, twice as long, came from L2 anew in every launch (138 instead of 121 us).
+// code, twice as long, came from L2 anew in every launch (17 us more at 64^3).
 
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>

@@ -421,8 +421,8 @@ __device__ __forceinline__ float fx_to_float(double x) {
 }
 
 // The FP32-output residual of k_outer_residual_v4 in the exact form above.  128^3
-// (3 components, with the norm): 69 us, bound by the integer pipe at 150
-// instructions per unknown; 84 us with 180 of them and the norm summed by FP64
+// (3 components, with the norm): 67 us, bound by the integer pipe at about 150
+// instructions per unknown; 82 us with 180 of them and the norm summed by FP64
 // shuffles in every warp of 256-thread blocks (a third of the FP64 work).
 constexpr int kFxBlock = 128;
 template <bool NORM>

@@ -10,7 +10,7 @@
 // (Algorithm 1) to a tolerance a hundred times tighter than the outer one:
 // with FP32 inner cycles on 3-D grids of a power of two up to 128, FP64
 // refinement around the spectral solve of the channel's operator, whose three
-// launches per iteration gain six digits (mobility at 64^3, 12 solves: 4.5 ms,
+// launches per iteration gain six digits (mobility at 64^3, 12 solves: 4.1 ms,
 // where their 99 FAC V-cycles took 20.5 ms); elsewhere FAC.  The Schur complement is symmetric positive semidefinite with
 // the constants as its kernel, and the right-hand side D(.) sums to zero, so
 // plain CG converges on the mean-free pressures; u is accumulated from the
