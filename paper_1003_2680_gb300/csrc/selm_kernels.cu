@@ -377,16 +377,21 @@ __device__ __forceinline__ long long fx_align(long long bits, int emax) {
 }
 
 // The same for a window of exponents within 31 of emax (none zero): one 64-bit
-// shift by less than 32.  A negative value -a is ~((a - 1) >> d), the same floor.
+// shift by less than 32.  A negative value -a is ~((a - 1) >> d), the same floor;
+// a = 32 m (- 1) as a wide multiply-add stays off the integer pipe, which bounds
+// the kernel (128^3: 65.2 us; 67.4 by shifts and adds, 66.4 by shifts alone with
+// the magnitude truncated).
 __device__ __forceinline__ unsigned long long fx_align31(long long bits, unsigned emax20) {
   const unsigned hi = (unsigned)((unsigned long long)bits >> 32), lo = (unsigned)bits;
   const unsigned sh = (emax20 - (hi & 0x7ff00000u)) >> 20;
   const unsigned mh = (hi & 0x000fffffu) | 0x00100000u;
-  const int s = (int)hi >> 31;   // all ones for a negative value
-  const unsigned long long a =
-      (((unsigned long long)__funnelshift_l(lo, mh, 5) << 32) | (lo << 5)) + (unsigned long long)(long long)s;
+  const unsigned s = (unsigned)((int)hi >> 31);   // all ones for a negative value
+  unsigned long long a;
+  asm("mad.wide.u32 %0, %1, 32, %2;"
+      : "=l"(a)
+      : "r"(lo), "l"(((unsigned long long)(32u * mh + s) << 32) | s));
   const unsigned ah = (unsigned)(a >> 32), al = (unsigned)a;
-  return ((unsigned long long)((ah >> sh) ^ (unsigned)s) << 32) | (__funnelshift_r(al, ah, sh) ^ (unsigned)s);
+  return ((unsigned long long)((ah >> sh) ^ s) << 32) | (__funnelshift_r(al, ah, sh) ^ s);
 }
 
 // S 2^e2 rounded to nearest even as FP64 (S != 0 and the result normal,
@@ -421,7 +426,7 @@ __device__ __forceinline__ float fx_to_float(double x) {
 }
 
 // The FP32-output residual of k_outer_residual_v4 in the exact form above.  128^3
-// (3 components, with the norm): 67 us, bound by the integer pipe at about 150
+// (3 components, with the norm): 65 us, bound by the integer pipe at about 150
 // instructions per unknown; 82 us with 180 of them and the norm summed by FP64
 // shuffles in every warp of 256-thread blocks (a third of the FP64 work).
 constexpr int kFxBlock = 128;
