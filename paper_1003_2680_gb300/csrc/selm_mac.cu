@@ -1205,7 +1205,7 @@ selm_status zero_mean(selm_mac* h, cudaStream_t st) {
 // The same conjugate gradients with the spectral solve of the composite
 // operator (FP32, selm_spectral.cu) as the preconditioner: exact up to FP32
 // rounding, so the FP64 recurrence gains five to seven digits per iteration
-// (64^3 + 8 rows to 1e-13: 3 iterations instead of 512, 0.65 ms instead of 18).
+// (64^3 + 8 rows to 1e-13: 3 iterations instead of 512, 0.58 ms instead of 18).
 // The residual and all inner products stay FP64.  It stops at proj_tol / 32, as far
 // below as the diagonal preconditioner got by testing every 16th iteration only:
 // stopping at proj_tol left errors of up to 6e-14 where that had 8e-15 to 4e-14
@@ -1246,15 +1246,18 @@ selm_status pressure_solve_spectral(selm_mac* h, const double* rhs, int* iters, 
         k_reduce<<<1, kThreads, 0, st>>>(h->part2, (int)nb, h->sc + old);
         MCK(cudaMemcpyAsync(h->cg_p, h->cg_z, n * sizeof(double), cudaMemcpyDeviceToDevice, st));
       } else {
-        k_cg_dir<<<nb, kThreads, 0, st>>>(n, (int)nb, h->part2, h->sc, old ^ 1, h->cg_z, h->cg_p);
+        MCK(launch_pdl(k_cg_dir, nb, kThreads, st, n, (int)nb, (const double*)h->part2, h->sc, old ^ 1,
+                       (const double*)h->cg_z, h->cg_p));
       }
-      k_cg_mv<<<nb, kThreads, 0, st>>>(h->S, h->cg_p, h->cg_q, h->part);
-      k_cg_update<false><<<nb, kThreads, 0, st>>>(n, (int)nb, h->part, h->sc, old, h->cg_x, h->cg_r, h->cg_p, h->cg_q,
-                                                  nullptr, nullptr, h->part2);
+      MCK(launch_pdl(k_cg_mv, nb, kThreads, st, h->S, (const double*)h->cg_p, h->cg_q, h->part));
+      MCK(launch_pdl(k_cg_update<false>, nb, kThreads, st, n, (int)nb, (const double*)h->part, (const double*)h->sc,
+                     old, h->cg_x, h->cg_r, (const double*)h->cg_p, (const double*)h->cg_q, (const double*)nullptr,
+                     (double*)nullptr, h->part2));
       k_reduce<<<1, kThreads, 0, st>>>(h->part2 + kRedBlocks, (int)nb, h->sc + 3);
       MCK(cudaGetLastError());
     }
     ++it;
+    if (it == 1 && tol < 1e-8) continue;   // out of reach of one FP32 solve: no host read before the second
     MCK(cudaMemcpyAsync(h->host_sc, h->sc, 8 * sizeof(double), cudaMemcpyDeviceToHost, st));
     MCK(cudaStreamSynchronize(st));
     const double rn_new = std::sqrt(h->host_sc[3]);
